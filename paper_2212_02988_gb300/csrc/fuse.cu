@@ -7,20 +7,7 @@
 
 namespace prism {
 
-template <bool BF16>
-__global__ void __launch_bounds__(256) k_fuse(KParams P, MapPlanes M, const float* __restrict__ w2c,
-                                              const float* __restrict__ depth, const float* __restrict__ rgb,
-                                              const uint8_t* __restrict__ mask, DevStats* __restrict__ stats) {
-    pdl_enter();
-    __shared__ float sM[9], sb[3];
-    load_w2c(w2c, sM, sb);
-    __syncthreads();
-    fuse_tile<BF16>(P, M, sM, sb, depth, rgb, mask, stats, blockIdx.x);
-}
-
-// The tiles in the frustum, appended to `list` (ctr[0] counts them; the
-// order is irrelevant: every tile's update is independent of the others).
-// rejected (nullable): a nonzero value lists no tile (the localisation of
+// The tiles in the frustum, appended to `list` (ctr[0] counts them).  rejected (nullable): a nonzero value lists no tile (the localisation of
 // this step was rejected, so its frame is not fused).
 __global__ void __launch_bounds__(256) k_fuse_cull(KParams P, const float* __restrict__ w2c, int* __restrict__ list,
                                                    unsigned int* __restrict__ ctr, const int* __restrict__ rejected) {
@@ -28,16 +15,7 @@ __global__ void __launch_bounds__(256) k_fuse_cull(KParams P, const float* __res
     __shared__ float sM[9], sb[3];
     load_w2c(w2c, sM, sb);
     __syncthreads();
-    const int n = P.nbx * P.nby * P.nbz;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    bool keep = false;
-    if (t < n && !(rejected && *rejected)) keep = !tile_outside_frustum(P, sM, sb, t % P.nbx, (t / P.nbx) % P.nby, t / (P.nbx * P.nby));
-    const unsigned int ballot = __ballot_sync(0xffffffffu, keep);
-    const int lane = threadIdx.x & 31;
-    unsigned int base = 0;
-    if (lane == 0 && ballot) base = atomicAdd(&ctr[0], (unsigned int)__popc(ballot));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (keep) list[base + __popc(ballot & ((1u << lane) - 1u))] = t;
+    cull_tiles(P, sM, sb, blockIdx.x * blockDim.x + threadIdx.x, rejected && *rejected, list, &ctr[0]);
 }
 
 // Persistent over the listed tiles; the last block to finish (ticket in
@@ -53,7 +31,7 @@ __global__ void __launch_bounds__(256, 4) k_fuse_list(KParams P, MapPlanes M, co
     __syncthreads();
     const unsigned int count = ctr[0];
     for (unsigned int i = blockIdx.x; i < count; i += gridDim.x) {
-        fuse_tile<BF16, false>(P, M, sM, sb, depth, rgb, mask, stats, (uint32_t)list[i]);
+        fuse_tile<BF16>(P, M, sM, sb, depth, rgb, mask, stats, (uint32_t)list[i]);
         __syncthreads();   // the tile's shared reduction scratch is reused by the next item
     }
     __shared__ int s_last;
@@ -91,16 +69,6 @@ cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float
                                   (const int*)list, ctr);
     return launch_pdl(k_fuse_list<false>, fuse_grid<false>(), 256, s, P, M, w2c, depth, rgb, mask, stats,
                       (const int*)list, ctr);
-}
-
-cudaError_t launch_fuse(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
-                        const float* rgb, const uint8_t* mask, DevStats* stats, cudaStream_t s) {
-    const unsigned int tiles = (unsigned int)(P.nbx * P.nby * P.nbz);
-    if (P.bf16)
-        launch_pdl(k_fuse<true>, tiles, 256, s, P, M, w2c, depth, rgb, mask, stats);
-    else
-        launch_pdl(k_fuse<false>, tiles, 256, s, P, M, w2c, depth, rgb, mask, stats);
-    return cudaGetLastError();
 }
 
 }  // namespace prism

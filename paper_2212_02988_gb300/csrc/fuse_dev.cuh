@@ -16,9 +16,9 @@
 // f_occ = -clamp(sdf, -trunc, trunc) (App. D: f_update = [-f_sdf, f_rgb]);
 // colour (one shared variance, reading R11) only where |sdf| <= trunc (R10).
 // A voxel outside the update region is not written (its occupancy is read
-// for the tile's bound), and a tile whose bounding sphere misses the view
-// frustum exits at once; every other tile refreshes its occupancy bounds
-// (kernels.h, MapPlanes::tb).
+// for the tile's bound).  Only tiles whose bounding sphere meets the view
+// frustum are updated (cull_tiles lists them); each refreshes its occupancy
+// bounds (kernels.h, MapPlanes::tb).
 #pragma once
 
 #include "kernels.h"
@@ -72,6 +72,22 @@ __device__ __forceinline__ bool tile_outside_frustum(const KParams& P, const flo
     return out;
 }
 
+// Tile t appended to `list` if it is in the frustum (count: its length; the
+// order is irrelevant, every tile's update being independent of the others).
+// Every thread of a warp calls it; none: list nothing.
+__device__ __forceinline__ void cull_tiles(const KParams& P, const float* sM, const float* sb, int t, bool none,
+                                           int* __restrict__ list, unsigned int* __restrict__ count) {
+    const int n = P.nbx * P.nby * P.nbz;
+    bool keep = false;
+    if (t < n && !none) keep = !tile_outside_frustum(P, sM, sb, t % P.nbx, (t / P.nbx) % P.nby, t / (P.nbx * P.nby));
+    const unsigned int ballot = __ballot_sync(0xffffffffu, keep);
+    const int lane = threadIdx.x & 31;
+    unsigned int base = 0;
+    if (lane == 0 && ballot) base = atomicAdd(count, (unsigned int)__popc(ballot));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (keep) list[base + __popc(ballot & ((1u << lane) - 1u))] = t;
+}
+
 // The world-to-camera matrices into shared memory (12 threads; the caller
 // synchronises before use).
 __device__ __forceinline__ void load_w2c(const float* __restrict__ w2c, float* sM, float* sb) {
@@ -81,22 +97,15 @@ __device__ __forceinline__ void load_w2c(const float* __restrict__ w2c, float* s
     }
 }
 
-// One 8x8x8 tile (256 threads); sM / sb: the world-to-camera matrices in
-// shared memory, loaded by the caller; CULL: test the frustum first (else the
-// caller has listed only tiles that pass it).
-template <bool BF16, bool CULL = true>
+// One 8x8x8 tile (256 threads) of those in the frustum; sM / sb: the
+// world-to-camera matrices in shared memory, loaded by the caller.
+template <bool BF16>
 __device__ __forceinline__ void fuse_tile(const KParams& P, const MapPlanes& M, const float* sM, const float* sb,
                                           const float* __restrict__ depth, const float* __restrict__ rgb,
                                           const uint8_t* __restrict__ mask, DevStats* __restrict__ stats,
                                           uint32_t tile) {
-    __shared__ int s_skip;
     if (!PRISM_IN_RANGE(P, CHK_FUSE_TILE, tile, (long long)P.nbx * P.nby * P.nbz)) return;   // block-uniform
     const int bx = tile % P.nbx, by = (tile / P.nbx) % P.nby, bz = tile / (P.nbx * P.nby);
-    if (CULL) {
-        if (threadIdx.x == 0) s_skip = tile_outside_frustum(P, sM, sb, bx, by, bz);
-        __syncthreads();
-        if (s_skip) return;
-    }
     const float fW1 = (float)(P.W - 1), fH1 = (float)(P.H - 1);
     unsigned int n_occ = 0, n_col = 0;
     // The thread's two voxels go through each stage together, so that each

@@ -124,12 +124,9 @@ cudaError_t launch_predict_prep(const KParams& P, DevState* dev, const double* i
                                 cudaStream_t s);
 
 // fuse.cu — the per-voxel map update with the world-to-camera matrices
-// `w2c` (12 FP32 on the device, DevState::w2c).
-cudaError_t launch_fuse(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
-                        const float* rgb, const uint8_t* mask, DevStats* stats, cudaStream_t s);
-// The same update in two launches: the frustum test of every tile appends
-// the tiles in view to `list` (ntiles ints), then a persistent grid updates
-// only those; ctr (2 uints, zero between calls) counts them.  rejected
+// `w2c` (12 FP32 on the device, DevState::w2c), in two launches: the frustum
+// test of every tile appends the tiles in view to `list` (ntiles ints), then
+// a persistent grid updates only those; ctr (2 uints, zero between calls) counts them.  rejected
 // (device int, nullable; DevState::rejected): nonzero lists no tile.
 cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
                                const float* rgb, const uint8_t* mask, DevStats* stats, int* list, unsigned int* ctr,

@@ -46,7 +46,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // Byte layout of one stream's single device allocation.
 struct StreamLayout {
     size_t plane, off_map, off_tb, off_bb, off_depth, off_rgb, off_omask, off_adepth, off_argb, off_a0, off_a1,
-        off_dev, off_stats, off_partials, off_counter, total;
+        off_dev, off_stats, off_partials, off_counter, off_list, total;
     int max_blocks;
 };
 
@@ -80,7 +80,8 @@ StreamLayout layout_of(const prism_config* c, int storage, int sms) {
     L.off_dev = take(sizeof(DevState));
     L.off_stats = take(sizeof(DevStats));
     L.off_partials = take((size_t)L.max_blocks * TRACK_NV_MAX * sizeof(float));
-    L.off_counter = take(sizeof(unsigned int));
+    L.off_counter = take(2 * sizeof(unsigned int));
+    L.off_list = take((size_t)kp.nbx * kp.nby * kp.nbz * sizeof(int));
     L.total = o;
     return L;
 }
@@ -233,6 +234,8 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
     d.a1 = (float4*)(b + L.off_a1);
     d.partials = (float*)(b + L.off_partials);
     d.counter = (unsigned int*)(b + L.off_counter);
+    d.fuse_count = d.counter + 1;
+    d.fuse_list = (int*)(b + L.off_list);
     d.pstride = L.max_blocks;
     d.grid_gn = track_launch_grid(st->kp, TRACK_GN, L.max_blocks);
     d.grid_lap = track_launch_grid(st->kp, TRACK_LAPLACE, L.max_blocks);
@@ -267,7 +270,7 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
     // pageable source: the copy is staged before the call returns
     if ((e = cudaMemcpyAsync(d.dev, &ds, sizeof(ds), cudaMemcpyHostToDevice, S->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(d.stats, 0, sizeof(DevStats), S->stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), S->stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(d.counter, 0, 2 * sizeof(unsigned int), S->stream)) != cudaSuccess) return e;
     PoseArg pa{};
     if ((e = launch_prep(d.dev, PREP_STATE, pa, S->stream)) != cudaSuccess) return e;
     *kernels += 1;
@@ -359,7 +362,7 @@ void run_batch(prism_server* S, std::unique_lock<std::mutex>& lk) {
         const int npix = st->kp.W * st->kp.H;
         B.tiles_off[i + 1] = B.tiles_off[i] + d.tiles_x * ((st->kp.H + 7) / 8);
         B.pix_off[i + 1] = B.pix_off[i] + (npix + 255) / 256;
-        B.fuse_off[i + 1] = B.fuse_off[i] + st->kp.nbx * st->kp.nby * st->kp.nbz;
+        B.cull_off[i + 1] = B.cull_off[i] + (st->kp.nbx * st->kp.nby * st->kp.nbz + 255) / 256;
         B.brick_off[i + 1] = B.brick_off[i] + st->kp.bb_len - st->kp.bb_off[st->kp.nlev];
         ups.push_back({d.depth, d.rgb, q.depth, q.rgb, (size_t)npix});
         fl.ids[i] = id;
@@ -400,7 +403,7 @@ void run_batch(prism_server* S, std::unique_lock<std::mutex>& lk) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(R.out, S->d_out, sizeof(ServeOut) * B.n, cudaMemcpyDeviceToHost, S->stream);
     if (e == cudaSuccess) e = cudaEventRecord(R.done, S->stream);
     lk.lock();
-    S->launches += 8 + n_gn;
+    S->launches += kServeKernels + n_gn;
     if (use_graph) S->graph_launches += 1;
     if (e != cudaSuccess) set_failed(S, std::string("batch launch: ") + cudaGetErrorString(e));
     S->cv_done.notify_all();   // wakes the completion thread

@@ -3,7 +3,7 @@
 //
 // A batch is a set of streams, one pending request each.  Every kernel of
 // the batched step is one persistent launch that walks the work items of all
-// members — 16x8 render tiles, 256-pixel blocks, 8^3 voxel tiles, virtual
+// members — 16x8 render tiles, 256-pixel blocks, listed 8^3 voxel tiles, virtual
 // blocks of the localisation passes — through prefix sums over the members,
 // and runs on each item the same device body as the single-stream kernel
 // (render_dev.cuh, track_dev.cuh, fuse_dev.cuh, state_dev.cuh).  The
@@ -39,6 +39,8 @@ struct SlotDesc {
     float4* a1;
     float* partials;           // localisation partials, value-major with stride pstride
     unsigned int* counter;     // ticket of the localisation passes
+    int* fuse_list;            // the tiles in this step's frustum (kb_cull)
+    unsigned int* fuse_count;  // how many; zero between batches
     int pstride;
     int grid_gn, grid_lap;     // virtual grids of the Gauss-Newton and Laplace passes
     int px_spec;               // render stride specialisation (render_px_specialisation)
@@ -61,7 +63,7 @@ struct BatchDesc {
     int loc[kServeMaxSlots];                // their member indices
     int tiles_off[kServeMaxSlots + 1];      // prefix sums over members: render tiles
     int pix_off[kServeMaxSlots + 1];        // 256-pixel blocks
-    int fuse_off[kServeMaxSlots + 1];       // 8^3 voxel tiles
+    int cull_off[kServeMaxSlots + 1];       // 256-tile groups of 8^3 voxel tiles
     int brick_off[kServeMaxSlots + 1];      // top-level bricks
     int gn_off[kServeMaxSlots + 1];         // over localising members: Gauss-Newton virtual blocks
     int lap_off[kServeMaxSlots + 1];        // Laplace virtual blocks
@@ -85,7 +87,9 @@ struct BatchGrids {
 
 cudaError_t batch_grids(bool bf16, BatchGrids* g);
 
-// Enqueues the batched step (8 + n_gn kernels) on s.
+constexpr int kServeKernels = 9;   // of a batched step beside its n_gn Gauss-Newton passes
+
+// Enqueues the batched step (kServeKernels + n_gn kernels) on s.
 cudaError_t launch_batch_step(const SlotDesc* slots, BatchDesc* batch, const double* imu, ServeOut* out, int n_gn,
                               bool bf16, const BatchGrids& g, cudaStream_t s);
 
