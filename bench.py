@@ -568,7 +568,7 @@ def run_ours(args, rank, world, local_rank):
                                                  "2 x 8 x 3 x %d B, per launch" % (b, b, b, b),
                             "unique_bytes_per_launch": U, "gathered_bytes_per_launch": G,
                             "samples_per_launch": samp_per, "ms_per_launch": render_ms},
-        "roofline_fuse": {"kernel": "k_fuse_cull + k_fuse_list + k_brick_bounds (the map-update phase)",
+        "roofline_fuse": {"kernel": "k_fuse_cull + k_fuse_list + k_brick_flags + k_box_codes (the map-update phase)",
                           "bound": "latency (dependent pixel, map and store round trips per tile; the listed "
                                    "tiles' occupancy read for their bounds)",
                           "achieved": fuse_bytes / (fuse_ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",

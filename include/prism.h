@@ -78,7 +78,7 @@ typedef struct {
     int32_t storage;             /* PRISM_STORAGE_F32 or PRISM_STORAGE_BF16 (map means and variances) */
     int32_t width, height;       /* frame size, pixels (>= 3 each) */
     int32_t n_gn;                /* Gauss-Newton iterations per frame (>= 1) */
-    int32_t skip_empty;          /* 1: rays skip 4^3 bricks whose occupancy bound stays below tau
+    int32_t skip_empty;          /* 1: rays skip 4^3 bricks whose occupancy stays below tau
                                     (same outputs, fewer samples); 0: every sample is evaluated */
     double voxel;                /* voxel edge length vs, metres */
     double origin[3];            /* world position of the grid's minimum corner */
@@ -376,7 +376,7 @@ prism_status prism_set_cooperative(prism_handle h, int32_t enabled);
 
 /* Bounds-check build.  libprism_checked.so is this library compiled with
  * PRISM_CHECKED: its kernels test the data-dependent index of every gather
- * and scatter (a trilinear cell's last corner in a map plane, a brick bound,
+ * and scatter (a trilinear cell's last corner in a map plane, a box of the empty-space index,
  * an anchor gather of the localisation, a block's partial column, a listed
  * fuse tile, a voxel and its nearest pixel in the map update, a corner of the
  * render adjoint, a tile of the anchor render's order) before the access, skip
@@ -384,7 +384,7 @@ prism_status prism_set_cooperative(prism_handle h, int32_t enabled);
  * prism_checked_build returns 1 in that library, 0 in libprism.so.
  * prism_check_status synchronises the handle's stream and writes its first
  * violation to *word: 0 for none, else (site << 48) | (index & (2^48 - 1)),
- * site 1 render corner, 2 brick bound, 3 anchor gather, 4 partial column,
+ * site 1 render corner, 2 empty-space box, 3 anchor gather, 4 partial column,
  * 5 fuse tile, 6 fuse voxel, 7 fuse pixel, 8 adjoint corner, 9 tile order;
  * always 0 in libprism.so, whose kernels carry no tests.  A violation means
  * a wrong result, never an access outside a buffer.  PRISM_EINVAL for a

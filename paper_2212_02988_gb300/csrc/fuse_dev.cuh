@@ -15,10 +15,10 @@
 // which is Lambda' = Lambda + Lu, mu' = (Lambda mu + Lu f) / Lambda'.
 // f_occ = -clamp(sdf, -trunc, trunc) (App. D: f_update = [-f_sdf, f_rgb]);
 // colour (one shared variance, reading R11) only where |sdf| <= trunc (R10).
-// A voxel outside the update region is not written (its occupancy is read
-// for the tile's bound).  Only tiles whose bounding sphere meets the view
-// frustum are updated (cull_tiles lists them); each refreshes its occupancy
-// bounds (kernels.h, MapPlanes::tb).
+// A voxel outside the update region is not written.  Only tiles whose bounding
+// sphere meets the view frustum are updated (cull_tiles lists them); the
+// empty-space index of the render is refreshed by a kernel that follows
+// (brick_flags_tiles).
 #pragma once
 
 #include "kernels.h"
@@ -47,15 +47,16 @@ __device__ void store_ghosts(const KParams& P, void* plane, int x, int y, int z,
 
 }  // namespace fuse_detail
 
-// Conservative frustum cull of tile (bx, by, bz): its bounding sphere
-// (centre c, radius r, with a margin far above FP32 rounding) lies entirely
-// behind the camera or outside a side plane of the pixel range
-// u, v in [-1/2, W - 1/2) x [-1/2, H - 1/2).  sM / sb: world-to-camera.
-__device__ __forceinline__ bool tile_outside_frustum(const KParams& P, const float* sM, const float* sb, int bx,
-                                                     int by, int bz) {
-    const float h = 4.0f * P.vs32;
-    const float cw[3] = {P.o32[0] + (8 * bx + 4) * P.vs32, P.o32[1] + (8 * by + 4) * P.vs32,
-                         P.o32[2] + (8 * bz + 4) * P.vs32};
+// Conservative frustum cull of the cube of `tiles` 8^3 tiles a side whose
+// lowest tile is (bx, by, bz): its bounding sphere (centre c, radius r, with a
+// margin far above FP32 rounding) lies entirely behind the camera or outside a
+// side plane of the pixel range u, v in [-1/2, W - 1/2) x [-1/2, H - 1/2).
+// sM / sb: world-to-camera.
+__device__ __forceinline__ bool outside_frustum(const KParams& P, const float* sM, const float* sb, int bx, int by,
+                                                int bz, int tiles) {
+    const float half = 4.0f * (float)tiles, h = half * P.vs32;
+    const float cw[3] = {P.o32[0] + (8 * bx + half) * P.vs32, P.o32[1] + (8 * by + half) * P.vs32,
+                         P.o32[2] + (8 * bz + half) * P.vs32};
     float c[3];
     for (int r = 0; r < 3; ++r) c[r] = sM[3 * r] * cw[0] + sM[3 * r + 1] * cw[1] + sM[3 * r + 2] * cw[2] + sb[r];
     const float rad = 1.7321f * h * 1.001f + 1e-4f;
@@ -72,20 +73,33 @@ __device__ __forceinline__ bool tile_outside_frustum(const KParams& P, const flo
     return out;
 }
 
-// Tile t appended to `list` if it is in the frustum (count: its length; the
-// order is irrelevant, every tile's update being independent of the others).
-// Every thread of a warp calls it; none: list nothing.
-__device__ __forceinline__ void cull_tiles(const KParams& P, const float* sM, const float* sb, int t, bool none,
-                                           int* __restrict__ list, unsigned int* __restrict__ count) {
-    const int n = P.nbx * P.nby * P.nbz;
-    bool keep = false;
-    if (t < n && !none) keep = !tile_outside_frustum(P, sM, sb, t % P.nbx, (t / P.nbx) % P.nby, t / (P.nbx * P.nby));
+// t appended to `list` (count: its length) on the lanes that keep it; the
+// order is irrelevant.  Every thread of a warp calls it.
+__device__ __forceinline__ void append_kept(bool keep, int t, int* __restrict__ list, unsigned int* __restrict__ count) {
     const unsigned int ballot = __ballot_sync(0xffffffffu, keep);
     const int lane = threadIdx.x & 31;
     unsigned int base = 0;
     if (lane == 0 && ballot) base = atomicAdd(count, (unsigned int)__popc(ballot));
     base = __shfl_sync(0xffffffffu, base, 0);
     if (keep) list[base + __popc(ballot & ((1u << lane) - 1u))] = t;
+}
+
+// Tile t appended to `list` (count[0]) if it is in the frustum, and to
+// cells_list (nullable; count[1]) if one of its cells may read a voxel of a
+// tile in `list`: those are the tiles t whose cube t + {0, 1}^3 meets the
+// frustum (its sphere holds the spheres of its 8 tiles).  none: list nothing.
+__device__ __forceinline__ void cull_tiles(const KParams& P, const float* sM, const float* sb, int t, bool none,
+                                           int* __restrict__ list, int* __restrict__ cells_list,
+                                           unsigned int* __restrict__ count) {
+    const int n = P.nbx * P.nby * P.nbz;
+    bool keep = false, cells = false;
+    if (t < n && !none) {
+        const int bx = t % P.nbx, by = (t / P.nbx) % P.nby, bz = t / (P.nbx * P.nby);
+        keep = !outside_frustum(P, sM, sb, bx, by, bz, 1);
+        cells = cells_list && !outside_frustum(P, sM, sb, bx, by, bz, 2);
+    }
+    append_kept(keep, t, list, count);
+    if (cells_list) append_kept(cells, t, cells_list, count + 1);
 }
 
 // The world-to-camera matrices into shared memory (12 threads; the caller
@@ -112,8 +126,8 @@ __device__ __forceinline__ void fuse_tile(const KParams& P, const MapPlanes& M, 
     // stage's loads are in flight at once: (1) decisions up to the pixel, and
     // the pixel's mask and depth; (2) the update decision, and the map values
     // (and observed colour) of the voxels updated; (3) the updates.  The
-    // occupancy of every voxel is read in (1) for the tile's bounds, which
-    // take the value each voxel holds after the update.
+    // occupancy is read in (1) already: nearly every listed tile updates most
+    // of its voxels, and the load then waits beside the pixel's.
     int x[2], y[2], z[2], pix[2];
     uint32_t idx[2];
     float X2[2], dep[2], mu[2];
@@ -187,9 +201,8 @@ __device__ __forceinline__ void fuse_tile(const KParams& P, const MapPlanes& M, 
         const float mu1 = fmaf(vl, f, mu[h]) * inv, var1 = var[h] * inv;
         map_store<BF16>(M.occ, idx[h], mu1);
         map_store<BF16>(M.var_occ, idx[h], var1);
-        mu[h] = map_round<BF16>(mu1);
         if (edge) {
-            fuse_detail::store_ghosts<BF16>(P, M.occ, x[h], y[h], z[h], mu[h]);
+            fuse_detail::store_ghosts<BF16>(P, M.occ, x[h], y[h], z[h], map_round<BF16>(mu1));
             fuse_detail::store_ghosts<BF16>(P, M.var_occ, x[h], y[h], z[h], map_round<BF16>(var1));
         }
         ++n_occ;
@@ -210,12 +223,6 @@ __device__ __forceinline__ void fuse_tile(const KParams& P, const MapPlanes& M, 
             }
             ++n_col;
         }
-    }
-    // the occupancy bounds of the tile's 4^3 sub-tiles after this update (the
-    // render's brick skipping)
-    {
-        const float am[2] = {fabsf(mu[0]), fabsf(mu[1])};
-        subtile_bounds_store(P, M.tb, bx, by, bz, mu, am);
     }
     if (stats) {
         unsigned int a = (unsigned int)warp_sum_u64(n_occ), b = (unsigned int)warp_sum_u64(n_col);

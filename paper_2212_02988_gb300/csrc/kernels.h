@@ -35,13 +35,12 @@ struct MapPlanes {
     void* b;
     void* var_occ;
     void* var_rgb;
-    // per 4^3 sub-tile: (max occupancy mean, max |occupancy mean|) over its
-    // voxels, kept current by the fuse and by map fill / load; per 4^3 brick b
-    // (the cells whose lower corner lies in sub-tile b): the same over
-    // sub-tiles b + {0, 1}^3, derived from tb by launch_brick_bounds
-    // (render_dev.cuh)
-    float2* tb;
-    float2* bb;
+    // the empty-space index of the rays (render_dev.cuh), derived from the
+    // occupancy plane by launch_brick_flags and launch_box_codes: per 8^3 tile
+    // the 4^3 bricks of its cells that may hold a hit, and per 8^3 box (the
+    // same, in the order of box_index) those flags with the empty box around it
+    uint8_t* bricks;
+    uint16_t* boxes;
 };
 
 // The tile order of an anchor render and what the next one is planned from
@@ -125,12 +124,15 @@ cudaError_t launch_predict_prep(const KParams& P, DevState* dev, const double* i
 
 // fuse.cu — the per-voxel map update with the world-to-camera matrices
 // `w2c` (12 FP32 on the device, DevState::w2c), in two launches: the frustum
-// test of every tile appends the tiles in view to `list` (ntiles ints), then
-// a persistent grid updates only those; ctr (2 uints, zero between calls) counts them.  rejected
-// (device int, nullable; DevState::rejected): nonzero lists no tile.
+// test of every tile appends the tiles in view to `list`, then a persistent
+// grid updates only those; ctr[0] (zero between calls) counts them.  With
+// cells_list the test also appends the tiles whose cells may read an updated
+// voxel to it, counted by ctr[1] (for launch_brick_flags).  Each list
+// has room for every tile.  rejected (device int, nullable;
+// DevState::rejected): nonzero lists no tile.
 cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
-                               const float* rgb, const uint8_t* mask, DevStats* stats, int* list, unsigned int* ctr,
-                               const int* rejected, cudaStream_t s);
+                               const float* rgb, const uint8_t* mask, DevStats* stats, int* list, int* cells_list,
+                               unsigned int* ctr, const int* rejected, cudaStream_t s);
 
 // mapio.cu — fill with the prior, and conversion between the caller's dense
 // layout and the padded (ghost-bordered) device layout.
@@ -144,10 +146,15 @@ cudaError_t launch_map_store(const KParams& P, const MapPlanes& M, float* occ, f
 // d0, d1 (n0, n1 floats) by the SMs' loads; a plain launch of `blocks`.
 cudaError_t launch_frame_upload(const float* s0, float* d0, size_t n0, const float* s1, float* d1, size_t n1,
                                 int blocks, cudaStream_t s);
-// The tile bounds M.tb of the whole map (after a fill or a load), and the
-// brick bounds M.bb derived from them (after any change of M.tb).
-cudaError_t launch_tile_bounds(const KParams& P, const MapPlanes& M, cudaStream_t s);
-cudaError_t launch_brick_bounds(const KParams& P, const MapPlanes& M, cudaStream_t s);
+// The empty-space index (MapPlanes::bricks, boxes): the brick flags of the
+// count[0] tiles of `list` (after a map update) or, without a list, of every
+// tile of the map (after a fill or a load), then the box codes, which launch_box_codes derives
+// from the flags after any change of them; it also clears the two list
+// counters ctr (nullable).  launch_map_index: both, for the whole map.
+cudaError_t launch_brick_flags(const KParams& P, const MapPlanes& M, const int* list, const unsigned int* count,
+                               cudaStream_t s);
+cudaError_t launch_box_codes(const KParams& P, const MapPlanes& M, unsigned int* ctr, cudaStream_t s);
+cudaError_t launch_map_index(const KParams& P, const MapPlanes& M, cudaStream_t s);
 
 // rollout.cu — predictive rollouts (App. I): per candidate sequence one block
 // chains k predictions (App. E.1/E.2) from the posterior of `src` on its own
@@ -177,7 +184,7 @@ cudaError_t launch_render_frames(const KParams& P, const float* mats, int frames
 // the loss terms are added to *loss.  launch_map_step: mu <- mu - lr (g +
 // (mu - mu0) / prior_var) on every padded element of the occupancy (g_occ, N
 // floats) and colour (g_rgb, 3N floats, linear layout) planes, the prior
-// term of the loss added to *loss; the tile and brick bounds are left to the
+// term of the loss added to *loss; the empty-space index is left to the
 // caller.
 cudaError_t launch_map_loss(const KParams& P, float* depth, float* rgb, const uint8_t* mask, const float* obs_d,
                             const float* obs_c, double sd, double sc, double* loss, cudaStream_t s);

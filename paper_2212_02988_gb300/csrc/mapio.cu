@@ -60,29 +60,24 @@ __global__ void k_map_store(KParams P, MapPlanes M, float* __restrict__ occ, flo
     }
 }
 
-// One block per 8^3 tile: (max, max |.|) of the occupancy means of each of
-// its 4^3 sub-tiles.
+// The empty-space index (render_dev.cuh): the brick flags of each 8^3 tile of
+// the map or of the listed ones, two a block; then the box codes, one block per
+// 32^3 box.
 template <bool BF16>
-__global__ void __launch_bounds__(256) k_tile_bounds(KParams P, MapPlanes M) {
+__global__ void __launch_bounds__(256) k_brick_flags(KParams P, MapPlanes M, const int* __restrict__ list,
+                                                     const unsigned int* __restrict__ count) {
     pdl_enter();
-    const uint32_t tile = blockIdx.x;
-    const int bx = tile % P.nbx, by = (tile / P.nbx) % P.nby, bz = tile / (P.nbx * P.nby);
-    float m[2], a[2];
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int within = threadIdx.x + 256 * half;
-        m[half] = map_load<BF16>(M.occ, pad_index(P, bx * 8 + (within & 7), by * 8 + ((within >> 3) & 7),
-                                                  bz * 8 + (within >> 6)));
-        a[half] = fabsf(m[half]);
+    const unsigned int n = list ? *count : (unsigned int)(P.nbx * P.nby * P.nbz);
+    for (unsigned int i = 2 * blockIdx.x; i < n; i += 2 * gridDim.x) {
+        const unsigned int j = i + (threadIdx.x >> 7);
+        render_detail::brick_flags_tiles<BF16>(P, M, j < n ? (list ? list[j] : (int)j) : -1);
     }
-    subtile_bounds_store(P, M.tb, bx, by, bz, m, a);
 }
 
-// One block per top-level brick: the brick bounds of every level below it
-// (render_dev.cuh).
-__global__ void __launch_bounds__(512) k_brick_bounds(KParams P, MapPlanes M) {
+__global__ void __launch_bounds__(256) k_box_codes(KParams P, MapPlanes M, unsigned int* ctr) {
     pdl_enter();
-    render_detail::brick_pyramid_block(P, M, blockIdx.x);
+    if (ctr && blockIdx.x == 0 && threadIdx.x < 2) ctr[threadIdx.x] = 0u;
+    render_detail::box_codes_block(P, M, blockIdx.x);
 }
 
 static unsigned int io_grid(uint32_t n) {
@@ -157,18 +152,20 @@ cudaError_t launch_frame_upload(const float* s0, float* d0, size_t n0, const flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_tile_bounds(const KParams& P, const MapPlanes& M, cudaStream_t s) {
-    const unsigned int tiles = (unsigned int)(P.nbx * P.nby * P.nbz);
-    if (P.bf16) launch_pdl(k_tile_bounds<true>, tiles, 256, s, P, M);
-    else launch_pdl(k_tile_bounds<false>, tiles, 256, s, P, M);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_brick_bounds(P, M, s);
+cudaError_t launch_brick_flags(const KParams& P, const MapPlanes& M, const int* list, const unsigned int* count,
+                               cudaStream_t s) {
+    const int need = (P.nbx * P.nby * P.nbz + 1) / 2, grid = need < 152 * 8 ? need : 152 * 8;
+    return P.bf16 ? launch_pdl(k_brick_flags<true>, grid, 256, s, P, M, list, count)
+                  : launch_pdl(k_brick_flags<false>, grid, 256, s, P, M, list, count);
 }
 
-cudaError_t launch_brick_bounds(const KParams& P, const MapPlanes& M, cudaStream_t s) {
-    const unsigned int top = (unsigned int)(P.bb_len - P.bb_off[P.nlev]);
-    return launch_pdl(k_brick_bounds, top, 512, s, P, M);
+cudaError_t launch_box_codes(const KParams& P, const MapPlanes& M, unsigned int* ctr, cudaStream_t s) {
+    return launch_pdl(k_box_codes, P.ntx * P.nty * P.ntz, 256, s, P, M, ctr);
+}
+
+cudaError_t launch_map_index(const KParams& P, const MapPlanes& M, cudaStream_t s) {
+    cudaError_t e = launch_brick_flags(P, M, nullptr, nullptr, s);
+    return e != cudaSuccess ? e : launch_box_codes(P, M, nullptr, s);
 }
 
 }  // namespace prism

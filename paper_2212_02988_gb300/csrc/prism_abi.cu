@@ -69,24 +69,13 @@ void fill_kparams(const prism_config* c, KParams& k) {
     k.W = c->width; k.H = c->height;
     k.bf16 = c->storage == PRISM_STORAGE_BF16;
     k.skip = c->skip_empty;
-    // brick levels: level l + 1 halves level l's brick counts while all three are even
-    {
-        int dx = c->nx / 4, dy = c->ny / 4, dz = c->nz / 4, off = 0;
-        k.nlev = 0;
-        for (int l = 0;; ++l) {
-            k.bb_off[l] = off;
-            off += dx * dy * dz;
-            if (l == 3 || ((dx | dy | dz) & 1)) break;
-            dx /= 2; dy /= 2; dz /= 2;
-            k.nlev = l + 1;
-        }
-        k.bb_len = off;
-    }
+    k.ntx = (k.nbx + 3) / 4; k.nty = (k.nby + 3) / 4; k.ntz = (k.nbz + 3) / 4;
+    k.nbox = 64 * k.ntx * k.nty * k.ntz;
     // the march cannot take more than (nx + ny + nz) vs / eps in-grid samples
     double kcap = 2.0 * (c->nx + c->ny + c->nz) * c->voxel / c->eps + 2.0;
     double kuser = c->max_depth > 0 ? std::floor(c->max_depth / c->eps) : kcap;
     double km = kuser < kcap ? kuser : kcap;
-    k.kmax = km > 2.0e9 ? 2000000000 : (int)km;
+    k.kmax = km > 16777214.0 ? 16777214 : (int)km;   // (float)(kmax + 2) is exact: the march counts in floats
     for (int a = 0; a < 3; ++a) { k.o32[a] = (float)c->origin[a]; k.origin[a] = c->origin[a]; }
     k.vs32 = (float)c->voxel;
     k.inv_vs32 = (float)(1.0 / c->voxel);
@@ -527,18 +516,23 @@ prism_status do_fuse(prism_handle h, const float* depth, const float* rgb, bool 
     PhaseTimer t(h, PH_FUSE);
     if (!mask_ready) LAUNCH(h, launch_depth_mask(h->kp, depth, h->o_mask, h->stream), "observation mask");
     // after a localisation in the same step (mask_ready), a rejected step fuses nothing
+    const size_t tiles = (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz;
+    int* cells_list = h->kp.skip ? h->fuse_list + tiles : nullptr;
     LAUNCH(h, launch_fuse_listed(h->kp, h->map, h->dstate->w2c, depth, rgb, h->o_mask, h->dstats, h->fuse_list,
-                                 h->fuse_ctr, mask_ready ? &h->dstate->rejected : nullptr, h->stream),
+                                 cells_list, h->fuse_ctr, mask_ready ? &h->dstate->rejected : nullptr, h->stream),
            "fuse");
     ++h->launches;   // (two kernels: the frustum list and the update)
     if (h->kp.skip) {
         // the tile order is done long before (it started with the map update):
-        // waiting here keeps the brick bounds and the render back to back
+        // waiting here keeps the empty-space index and the render back to back
         if (h->plan_fresh && !h->plan_waited) {
             CK(h, cudaStreamWaitEvent(h->stream, h->ev_plan, 0), "wait for the tile order");
             h->plan_waited = true;
         }
-        LAUNCH(h, launch_brick_bounds(h->kp, h->map, h->stream), "brick bounds");
+        LAUNCH(h, launch_brick_flags(h->kp, h->map, cells_list, h->fuse_ctr + 1, h->stream), "brick flags");
+        LAUNCH(h, launch_box_codes(h->kp, h->map, h->fuse_ctr, h->stream), "box codes");
+    } else {
+        CK(h, cudaMemsetAsync(h->fuse_ctr, 0, 2 * sizeof(unsigned int), h->stream), "clear list counters");
     }
     return PRISM_OK;
 }
@@ -718,13 +712,13 @@ prism_status prism_create_map(const prism_config* cfg, const prism_state* s1, vo
         delete h;
         return fail(nullptr, st, m);
     };
-    const size_t tbytes = ((8 * (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz * sizeof(float2) + 255) / 256) * 256;
-    const size_t bbytes = (((size_t)h->kp.bb_len * sizeof(float2) + 255) / 256) * 256;
-    if (dalloc(h, &h->map_block, 6 * plane + tbytes + bbytes) != cudaSuccess)
+    const size_t cbytes = (((size_t)h->kp.nbx * h->kp.nby * h->kp.nbz + 255) / 256) * 256;
+    const size_t xbytes = (size_t)h->kp.nbox * sizeof(uint16_t);
+    if (dalloc(h, &h->map_block, 6 * plane + cbytes + xbytes) != cudaSuccess)
         return cleanup(PRISM_ENOMEM, "map allocation failed");
     char* base = (char*)h->map_block;
-    h->map.tb = (float2*)(base + 6 * plane);
-    h->map.bb = (float2*)(base + 6 * plane + tbytes);
+    h->map.bricks = (uint8_t*)(base + 6 * plane);
+    h->map.boxes = (uint16_t*)(base + 6 * plane + cbytes);
     h->map.occ = base;
     h->map.r = base + plane;
     h->map.g = base + 2 * plane;
@@ -736,7 +730,7 @@ prism_status prism_create_map(const prism_config* cfg, const prism_state* s1, vo
         dalloc(h, &h->dstate, sizeof(DevState)) || dalloc(h, &h->dstats, sizeof(DevStats)) ||
         dalloc(h, &h->partials, 2 * (size_t)h->max_blocks * TRACK_NV_MAX * sizeof(float)) ||
         dalloc(h, &h->counter, 2 * sizeof(unsigned int)) ||
-        dalloc(h, &h->fuse_list, (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz * sizeof(int)) ||
+        dalloc(h, &h->fuse_list, 2 * (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz * sizeof(int)) ||
         dalloc(h, &h->fuse_ctr, 2 * sizeof(unsigned int)))
         return cleanup(PRISM_ENOMEM, "device allocation failed");
     {   // tile costs, order and scratch (one word each per 16x8 tile), the rotation
@@ -774,7 +768,7 @@ prism_status prism_create_map(const prism_config* cfg, const prism_state* s1, vo
     }
     if ((e = launch_map_fill(h->kp, h->map, (float)cfg->init_occ, (float)cfg->init_rgb, (float)cfg->prior_var,
                              h->stream)) != cudaSuccess ||
-        (e = launch_tile_bounds(h->kp, h->map, h->stream)) != cudaSuccess)
+        (e = launch_map_index(h->kp, h->map, h->stream)) != cudaSuccess)
         return cleanup(PRISM_ECUDA, std::string("map fill: ") + cudaGetErrorString(e));
     if ((e = cudaMemsetAsync(h->dstats, 0, sizeof(DevStats), h->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(h->counter, 0, 2 * sizeof(unsigned int), h->stream)) != cudaSuccess ||
@@ -993,8 +987,8 @@ prism_status prism_map_load(prism_handle h, const float* occ, const float* rgb, 
     DeviceGuard g(h->device);
     LAUNCH(h, launch_map_load(h->kp, h->map, occ, rgb, var_occ, var_rgb, h->stream), "map load");
     if (occ) {
-        LAUNCH(h, launch_tile_bounds(h->kp, h->map, h->stream), "tile bounds");
-        ++h->launches;   // and the brick bounds derived from them
+        LAUNCH(h, launch_map_index(h->kp, h->map, h->stream), "empty-space index");
+        ++h->launches;   // (two kernels: the brick flags and the box codes)
     }
     return PRISM_OK;
 }
@@ -1167,8 +1161,8 @@ prism_status prism_map_descent(prism_handle h, int32_t n, const double* poses, c
     LAUNCH(h, launch_map_step(h->kp, h->map, g_occ, g_rgb, lr_occ, lr_rgb, h->cfg.init_occ, h->cfg.init_rgb,
                               h->cfg.prior_var, d_loss, h->stream),
            "descent step");
-    LAUNCH(h, launch_tile_bounds(h->kp, h->map, h->stream), "tile bounds");
-    ++h->launches;   // and the brick bounds derived from them
+    LAUNCH(h, launch_map_index(h->kp, h->map, h->stream), "empty-space index");
+    ++h->launches;   // (two kernels: the brick flags and the box codes)
     if (!loss) return PRISM_OK;
     CK(h, cudaMemcpyAsync(loss, d_loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream), "read loss");
     CK(h, cudaStreamSynchronize(h->stream), "stream synchronize");

@@ -5,13 +5,12 @@
 
 namespace prism {
 
-// Without DETAIL counters the march takes two samples a step (render_tile's
-// NS): 8 blocks an SM (64 registers) with two samples' loads in flight beat
-// 10 blocks with one, on the rays that march longest.  One block per 16x8
-// tile, block b rendering tile plan.order[b] (row-major without an order);
+// 6 blocks an SM (80 registers) with three samples' gathers in flight beat 8 (64)
+// here, where the longest rays set the time (8 in the rollouts, where the rate
+// does).  One block per 16x8 tile, block b rendering tile plan.order[b] (row-major without an order);
 // with plan.cost the block records the tile's cost for the next plan.
 template <bool BF16, bool DETAIL, int PX>
-__global__ void __launch_bounds__(128, DETAIL ? 10 : 8) k_render(KParams P, const float* __restrict__ mats, MapPlanes M,
+__global__ void __launch_bounds__(128, DETAIL ? 10 : 6) k_render(KParams P, const float* __restrict__ mats, MapPlanes M,
                                                 float* __restrict__ depth, float* __restrict__ rgb,
                                                 uint8_t* __restrict__ mask, int32_t* __restrict__ hitk,
                                                 DevStats* __restrict__ stats, const double* __restrict__ anchor_src,
@@ -35,8 +34,7 @@ __global__ void __launch_bounds__(128, DETAIL ? 10 : 8) k_render(KParams P, cons
         PRISM_IN_RANGE(P, CHK_PLAN, tile, nt);
         tile = (int)blockIdx.x;
     }
-    const int ns = render_tile<BF16, DETAIL, PX, DETAIL ? 1 : 2>(P, sR, sc, M, depth, rgb, mask, hitk, stats,
-                                                                   tile % gx, tile / gx);
+    const int ns = render_tile<BF16, DETAIL, PX>(P, sR, sc, M, depth, rgb, mask, hitk, stats, tile % gx, tile / gx);
     if (plan.cost) {
         const unsigned int wmax = __reduce_max_sync(0xffffffffu, (unsigned int)ns);
         if ((threadIdx.x & 31) == 0) atomicAdd(&s_cost, wmax);

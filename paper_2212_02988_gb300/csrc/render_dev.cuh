@@ -86,120 +86,392 @@ __device__ __forceinline__ Sample cell_of(uint32_t px, uint32_t pxy, float gx, f
     return s;
 }
 
-// Brick skipping.  A cell whose lower corner x0 lies in brick b = max(x0, 0) / 4
-// (per axis) reads corners from the 4^3 sub-tiles b and b + 1 only; brick_bound
-// is the bound of those 8 sub-tiles (MapPlanes::bb).  A trilinear value is a convex
-// combination of its corners, so if the bound is below tau by more than the
+// The empty-space index.  A trilinear value is a convex combination of its 8
+// corners, so a cell whose largest corner is below tau by more than the
 // lerps' rounding (7 lerps, each within ~3 2^-24 of the corners' magnitude:
-// 2^-18 (1 + max |corner|) is a safe margin), no sample in the brick can be a
-// hit and the march may jump over it.
-__device__ __forceinline__ float2 brick_bound(const KParams& P, const float2* __restrict__ tb, int bx, int by,
-                                              int bz) {
-    const int sx = 2 * P.nbx, sy = 2 * P.nby, sz = 2 * P.nbz;
-    const int bx1 = min(bx + 1, sx - 1), by1 = min(by + 1, sy - 1), bz1 = min(bz + 1, sz - 1);
-    float m = -INFINITY, a = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const int x = c & 1 ? bx1 : bx, y = c & 2 ? by1 : by, z = c & 4 ? bz1 : bz;
-        const float2 t = tb[x + sx * (y + sy * z)];
-        m = fmaxf(m, t.x);
-        a = fmaxf(a, t.y);
-    }
-    return make_float2(m, a);
+// 2^-18 (1 + max |corner|) is a safe margin) holds no sample that can be a
+// hit.  The index is 16 bits per 8^3 box of cells (those whose lower corner
+// lies in [8 b, 8 b + 8) per axis; a lower corner of -1 reads voxel 0 only,
+// which cell 0 reads too, and goes with cell 0):
+//   bits 0-7   the 4^3 bricks of the box with a cell that may hold a hit;
+//   bits 8-9   where there are none: c = 1, 2 or 3 for the largest aligned box
+//              around it, 4 2^c = 8, 16 or 32 cells a side, without any;
+//   bit 10     open: neither this box nor its 26 neighbours have any.
+// 64 KB for 256^3 voxels, 32 bytes for 32x32x8 of them (box_index): the rays'
+// lookups hit L1.
+//
+// How a warp's 32 rays use it.  First the warp goes together along the tile's
+// centre ray, each lane testing one distance for open boxes (beam_start): one
+// or two loads take all rays past the free space in front of the camera.
+// Then each ray jumps out of empty boxes and bricks on one load a jump, and
+// evaluates the samples in the remaining bricks, three at a time.  With 4^3
+// bounds of floats and three coarser levels of them (2.4 MB, two dependent
+// loads a jump), rays one by one from the camera, a frame took 38.2 us in a
+// launch of 320 (640x480, 256^3 map) and 55 us alone; now 22.4 and 37.6 us.
+constexpr uint32_t kBoxOpen = 1u << 10;
+
+// The word of box (x, y, z): the 4x4x4 boxes of a 32^3 box are consecutive.
+__device__ __forceinline__ int box_index(const KParams& P, int x, int y, int z) {
+    return 64 * ((x >> 2) + P.ntx * ((y >> 2) + P.nty * (z >> 2))) + ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
 }
 
-// The brick bounds below one top-level brick (level P.nlev, index `top`),
-// one 512-thread block: level 0 from the sub-tile bounds (brick_bound), level
-// l + 1 as the max of its 8 children at level l.  A level-l brick covers the
-// cells whose lower corner lies in its (4 * 2^l)^3 box, and each child bound
-// already includes the sub-tiles one step beyond it, so the max is the bound
-// of the sub-tiles those cells read.
-__device__ __forceinline__ void brick_pyramid_block(const KParams& P, const MapPlanes& M, int top) {
-    __shared__ float2 s_b[2][512];
-    const int N = P.nlev, s = 1 << N, t = threadIdx.x;
-    const int d0x = 2 * P.nbx, d0y = 2 * P.nby;
-    const int dNx = d0x >> N, dNy = d0y >> N;
-    const int Tx = top % dNx, Ty = (top / dNx) % dNy, Tz = top / (dNx * dNy);
-    if (t < s * s * s) {
-        const int x = Tx * s + t % s, y = Ty * s + (t / s) % s, z = Tz * s + t / (s * s);
-        const float2 b = brick_bound(P, M.tb, x, y, z);
-        M.bb[x + d0x * (y + d0y * z)] = b;
-        s_b[0][t] = b;
-    }
-    for (int l = 1; l <= N; ++l) {
-        __syncthreads();
-        const int sl = s >> l, sc = 2 * sl;   // level-l bricks and their children per axis in this block
-        if (t < sl * sl * sl) {
-            const int lx = t % sl, ly = (t / sl) % sl, lz = t / (sl * sl);
-            const float2* ch = s_b[(l - 1) & 1];
+// The flags of the 8 bricks of two 8^3 tiles (256 threads, 128 a tile; a
+// negative tile: none): a brick's cells read the 5^3 voxels from its lowest
+// one on, and it may hold a hit unless the largest of them is below tau as
+// above.  Warp w of a tile's four takes the layers z = 2 w .. 2 w + 2; its lane
+// l < 27 reads voxel x = l % 9 of the rows y = 3 i + l / 9: nine loads in flight
+// a lane.  Latency bound: 4.2 us for 512 tiles, 8.8 us for the ~3,400 of a
+// 640x480 step, 36 us for the 32,768 of a 256^3 map (a tile a block through
+// shared memory: 4.3, 10.3 and 75 us; a tile a warp: 9.4, 10.8 and 43).
+template <bool BF16>
+__device__ __forceinline__ void brick_flags_tiles(const KParams& P, const MapPlanes& M, int tile) {
+    __shared__ float2 s_b[2][4][4];   // [tile][warp][brick x + 2 y]: largest value and magnitude
+    const int t = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const bool on = tile >= 0 && PRISM_IN_RANGE(P, CHK_FUSE_TILE, tile, (long long)P.nbx * P.nby * P.nbz);
+    if (on) {
+        const int bx = tile % P.nbx, by = (tile / P.nbx) % P.nby, bz = tile / (P.nbx * P.nby);
+        const int l = lane < 27 ? lane : 26, x = l % 9, y0 = l / 9;
+        const uint32_t base = pad_index(P, 8 * bx + x, 8 * by + y0, 8 * bz + 2 * w);
+        float v[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) v[i] = map_load_rw<BF16>(M.occ, base + P.px * (3u * (i % 3)) + P.pxy * (i / 3));
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {   // y: 0 .. 4 (rows 3 r + y0), then 4 .. 8
             float m = -INFINITY, a = 0.0f;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float2 v = ch[(2 * lx + (c & 1)) + sc * ((2 * ly + ((c >> 1) & 1)) + sc * (2 * lz + (c >> 2)))];
-                m = fmaxf(m, v.x);
-                a = fmaxf(a, v.y);
+            for (int i = 0; i < 9; ++i) {
+                const int r = i % 3;
+                if (r == (q == 0 ? 2 : 0)) continue;
+                const bool in = r != 1 || (q == 0 ? y0 <= 1 : y0 >= 1);
+                m = fmaxf(m, in ? v[i] : -INFINITY);
+                a = fmaxf(a, in ? fabsf(v[i]) : 0.0f);
             }
-            const float2 r = make_float2(m, a);
-            const int dlx = d0x >> l, dly = d0y >> l;
-            M.bb[P.bb_off[l] + (Tx * sl + lx) + dlx * ((Ty * sl + ly) + dly * (Tz * sl + lz))] = r;
-            s_b[l & 1][t] = r;
+            // over the lanes' rows (l, l + 9, l + 18), then x = 0 .. 4 into lane 0 and 4 .. 8 into lane 4
+            auto reduce = [&](float z) {
+                const float r1 = __shfl_down_sync(0xffffffffu, z, 9), r2 = __shfl_down_sync(0xffffffffu, z, 18);
+                z = fmaxf(fmaxf(z, r1), r2);
+                const float s1 = fmaxf(z, __shfl_down_sync(0xffffffffu, z, 1));
+                const float s2 = fmaxf(s1, __shfl_down_sync(0xffffffffu, s1, 2));
+                return fmaxf(s2, __shfl_down_sync(0xffffffffu, z, 4));
+            };
+            m = reduce(m);
+            a = reduce(a);
+            if (lane == 0 || lane == 4) s_b[t][w][(lane >> 2) + 2 * q] = make_float2(m, a);
         }
     }
-    __syncthreads();   // the shared levels are reused by the block's next item
-}
-
-__device__ __forceinline__ bool brick_skippable(const KParams& P, const float2* __restrict__ bb, int brick) {
-    const float2 t = __ldg(bb + brick);
-    return t.x < P.tau32 - 0x1p-18f * (1.0f + t.y);
-}
-
-// The first sample index at or after which the ray may leave the level-lv
-// brick (bx, by, bz): the exit distance of its cell-corner box [e b, e b + e),
-// e = 4 * 2^lv (lower bound -1 for b = 0), pulled 1e-3 voxels inside, over
-// eps, plus one.  irg are the
-// reciprocals of the ray's grid direction (0 where it is 0) and ieps = 1 / eps;
-// the products stand in for the quotients, whose rounding (and that of the
-// sample positions) is far below the 1e-3 voxel margin.  Every sample before
-// the returned index has its cell in the brick.
-__device__ __forceinline__ int brick_exit(const KParams& P, int lv, int bx, int by, int bz, float irgx, float irgy,
-                                          float irgz, float cgx, float cgy, float cgz, float ieps) {
-    constexpr float m = 1e-3f;
-    const float e = (float)(4 << lv);
-    float dmin = INFINITY;
-    const int b3[3] = {bx, by, bz};
-    const float ir3[3] = {irgx, irgy, irgz}, cg3[3] = {cgx, cgy, cgz};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float lo = b3[a] == 0 ? -1.0f : e * (float)b3[a];
-        const float hi = e * (float)(b3[a] + 1);
-        if (ir3[a] > 0.0f) dmin = fminf(dmin, (hi - m - cg3[a]) * ir3[a]);
-        else if (ir3[a] < 0.0f) dmin = fminf(dmin, (lo + m - cg3[a]) * ir3[a]);
+    __syncthreads();
+    if (w == 0 && on) {   // lane: brick x + 2 y + 4 z
+        const float2 b0 = s_b[t][2 * ((lane >> 2) & 1)][lane & 3], b1 = s_b[t][2 * ((lane >> 2) & 1) + 1][lane & 3];
+        const uint32_t f = __ballot_sync(0xffffffffu, !(fmaxf(b0.x, b1.x) < P.tau32 - 0x1p-18f * (1.0f + fmaxf(b0.y, b1.y))));
+        if (lane == 0) M.bricks[tile] = (uint8_t)(f & 0xffu);
     }
-    const float kn = floorf(dmin * ieps) + 1.0f;
-    return kn < (float)(P.kmax + 1) ? (int)kn : P.kmax + 1;
+    __syncthreads();   // s_b is reused by the next tiles
+}
+
+// The words of the 64 boxes of one 32^3 box, one 256-thread block: the flags
+// of the 6^3 boxes around them go through shared memory; boxes past the map's
+// edge count as empty.
+__device__ __forceinline__ void box_codes_block(const KParams& P, const MapPlanes& M, int top) {
+    __shared__ uint8_t s_f[6][6][6];   // [z][y][x], the 32^3 box's own at 1 .. 4
+    __shared__ int s_all[2];
+    const int t = threadIdx.x;
+    const int x0 = 4 * (top % P.ntx), y0 = 4 * ((top / P.ntx) % P.nty), z0 = 4 * (top / (P.ntx * P.nty));
+    if (t < 216) {
+        const int i = t % 6, j = (t / 6) % 6, k = t / 36, x = x0 + i - 1, y = y0 + j - 1, z = z0 + k - 1;
+        s_f[k][j][i] = x >= 0 && x < P.nbx && y >= 0 && y < P.nby && z >= 0 && z < P.nbz
+                           ? M.bricks[x + P.nbx * (y + P.nby * z)] : (uint8_t)0;
+    }
+    __syncthreads();
+    uint32_t f = 0u, near = 0u;
+    int e1 = 0, e2 = 0;
+    if (t < 64) {   // box (t & 3, (t >> 2) & 3, t >> 4)
+        const int i = t & 3, j = (t >> 2) & 3, k = t >> 4;
+        f = s_f[k + 1][j + 1][i + 1];
+#pragma unroll
+        for (int c = 0; c < 27; ++c) near |= s_f[k + c / 9][j + (c / 3) % 3][i + c % 3];
+        e1 = f == 0u;
+        e2 = e1 & __shfl_xor_sync(0xffffffffu, e1, 1);   // the 2x2x2 boxes of its 16^3 box
+        e2 &= __shfl_xor_sync(0xffffffffu, e2, 4);
+        e2 &= __shfl_xor_sync(0xffffffffu, e2, 16);
+        const int all = __all_sync(0xffffffffu, e1);
+        if ((t & 31) == 0) s_all[t >> 5] = all;
+    }
+    __syncthreads();
+    if (t < 64) {
+        const uint32_t code = e1 ? (e2 ? (s_all[0] & s_all[1] ? 3u : 2u) : 1u) : 0u;
+        M.boxes[64 * (size_t)top + t] = (uint16_t)(f | (code << 8) | (near == 0u ? kBoxOpen : 0u));
+    }
+    __syncthreads();   // the shared flags are reused by the block's next item
+}
+
+// A ray in grid units: sample position g = fma(d, rg, cg), d = k eps.
+struct Ray {
+    float rx, ry, rz;      // unit world direction
+    float rgx, rgy, rgz, cgx, cgy, cgz;
+    float inv_n;           // 1 / |dir_c|
+};
+
+// The ray of pixel (u, v) (the FP32 recipe).
+__device__ __forceinline__ Ray ray_of(const KParams& P, const float* sR, const float* sc, int u, int v) {
+    Ray r;
+    const float dx = __fmul_rn(__fsub_rn((float)u, P.cx32), P.ifx32);
+    const float dy = __fmul_rn(__fsub_rn((float)v, P.cy32), P.ify32);
+    const float w0 = __fmaf_rn(sR[0], dx, __fmaf_rn(sR[1], dy, sR[2]));
+    const float w1 = __fmaf_rn(sR[3], dx, __fmaf_rn(sR[4], dy, sR[5]));
+    const float w2 = __fmaf_rn(sR[6], dx, __fmaf_rn(sR[7], dy, sR[8]));
+    r.inv_n = __fdiv_rn(1.0f, __fsqrt_rn(__fmaf_rn(w0, w0, __fmaf_rn(w1, w1, __fmul_rn(w2, w2)))));
+    r.rx = __fmul_rn(w0, r.inv_n);
+    r.ry = __fmul_rn(w1, r.inv_n);
+    r.rz = __fmul_rn(w2, r.inv_n);
+    r.rgx = __fmul_rn(r.rx, P.inv_vs32);
+    r.rgy = __fmul_rn(r.ry, P.inv_vs32);
+    r.rgz = __fmul_rn(r.rz, P.inv_vs32);
+    r.cgx = __fmaf_rn(__fsub_rn(sc[0], P.o32[0]), P.inv_vs32, -0.5f);
+    r.cgy = __fmaf_rn(__fsub_rn(sc[1], P.o32[1]), P.inv_vs32, -0.5f);
+    r.cgz = __fmaf_rn(__fsub_rn(sc[2], P.o32[2]), P.inv_vs32, -0.5f);
+    return r;
+}
+
+// One axis of a brick exit: the plane of the box's far side along the ray is
+// lo + s e + m (s = 1, m = -1e-3 for a positive direction; s = 0, m = 1e-3
+// for a negative one: pulled 1e-3 voxels inside, far above the rounding of
+// the sample positions and of the quotient; a zero direction: never), its
+// distance in samples (lo + s e + (m - cg)) / (rg eps).
+struct ExitAxis {
+    float s, c, ir;   // s; m - cg; 1 / (rg eps)
+    __device__ __forceinline__ ExitAxis(float rg, float cg, float ieps) {
+        s = rg > 0.0f ? 1.0f : 0.0f;
+        c = (rg > 0.0f ? -1e-3f : (rg < 0.0f ? 1e-3f : 1e30f)) - cg;
+        ir = rg != 0.0f ? ieps / rg : 1.0f;
+    }
+    // bits: the cell coordinate + kFloorMagicBits, clear: the bits below the box's
+    // edge, ef: the edge
+    __device__ __forceinline__ float dist(uint32_t bits, uint32_t clear, float ef) const {
+        const float lo = __uint_as_float(bits & ~clear) - kFloorMagic;   // exact
+        return (fmaf(s, ef, lo) + c) * ir;
+    }
+};
+
+// The sample index from which the 32 rays of a warp (all lanes call it, rays
+// or not) have to be marched: every sample before it lies in an open box or a
+// neighbour of one.  Lane j of a round tests the middle of the piece [j, j + 1)
+// S of the centre ray (unit direction rc), S = 8 voxels: a point of the piece
+// is at most 4 voxels from its middle on any axis, a ray's sample at the same
+// distance at most delta (j + 1) S more (delta: the largest difference of a
+// lane's direction from rc on any axis), together below the 8 voxels that an
+// open box has around it (0.1 voxel of margin, far above the rounding).  The
+// centre must be one voxel inside the grid (cg in [0.5, h - 1]): no sample
+// before the returned one has then left the grid and come back.
+__device__ __forceinline__ float beam_start(const KParams& P, const MapPlanes& M, const float* sR, const Ray& r, float uc,
+                                          float vc) {
+    const float hx = (float)P.nx - 1.5f, hy = (float)P.ny - 1.5f, hz = (float)P.nz - 1.5f;
+    if (!(r.cgx >= 0.5f && r.cgx <= hx && r.cgy >= 0.5f && r.cgy <= hy && r.cgz >= 0.5f && r.cgz <= hz)) return 1.0f;
+    const float dx = (uc - P.cx32) * P.ifx32, dy = (vc - P.cy32) * P.ify32;
+    float w0 = sR[0] * dx + sR[1] * dy + sR[2], w1 = sR[3] * dx + sR[4] * dy + sR[5], w2 = sR[6] * dx + sR[7] * dy + sR[8];
+    const float inv = rsqrtf(w0 * w0 + w1 * w1 + w2 * w2);
+    w0 *= inv;
+    w1 *= inv;
+    w2 *= inv;
+    const float dl = fmaxf(fmaxf(fabsf(r.rx - w0), fabsf(r.ry - w1)), fabsf(r.rz - w2));
+    // (a non-negative float's bits order as the float; 8 voxels a step)
+    const float delta = 8.0f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dl)));
+    const int lane = threadIdx.x & 31;
+    for (int base = 0;; base += 32) {
+        const float j = (float)(base + lane), s = 8.0f * (j + 0.5f);
+        const float gx = fmaf(s, w0, r.cgx), gy = fmaf(s, w1, r.cgy), gz = fmaf(s, w2, r.cgz);
+        bool open = (j + 1.0f) * delta <= 3.9f && gx >= 0.0f && gx <= hx && gy >= 0.0f && gy <= hy && gz >= 0.0f && gz <= hz;
+        if (open) {
+            const int bi = box_index(P, (int)gx >> 3, (int)gy >> 3, (int)gz >> 3);
+            open = PRISM_IN_RANGE(P, CHK_RENDER_BRICK, bi, P.nbox) && (__ldg(M.boxes + bi) & kBoxOpen) != 0u;
+        }
+        const uint32_t shut = ~__ballot_sync(0xffffffffu, open);
+        if (shut) {
+            const float d = 8.0f * (float)(base + __ffs(shut) - 1) * P.vs32;   // all samples before this distance
+            return fminf(fmaxf(floorf(d / P.eps32 * (1.0f - 1e-6f)), 1.0f), (float)P.kmax);
+        }
+    }
+}
+
+// What the march of a ray found: the index k of the first sample above tau (0:
+// none), its value and cell, and the value of sample k - 1 if it was evaluated.
+struct MarchHit {
+    int k;
+    float f, f_prev;
+    bool prev_ok;
+    Sample cur;
+};
+
+// The march of App. B: samples k = 1, 2, ... up to the first one above tau,
+// outside the grid or past kmax (below 2^24: fill_kparams; the index is a
+// float, exact there).  The grid bounds are tested only for samples after
+// k_safe, which a conservative FP32 bound (one voxel of margin, far above the
+// rounding of the bound and of the sample positions) keeps inside the grid.
+// With P.skip the empty-space index decides which samples are evaluated,
+// starting from k0 (beam_start); the hit and its values are those of the march
+// over every sample.  Every lane of the warp calls it (active: the lane has a
+// ray): the lanes jump until each has a sample to evaluate or has ended, then
+// evaluate together, NS samples from k on at once (8 NS gathers in flight), so
+// that a warp waits for its gathers a few times instead of whenever one lane
+// reaches a surface (a rollout's frame 27.6, 23.5, 22.4 and 23.2 us with NS = 1,
+// 2, 3, 4).  A later sample past kmax or outside the grid is ignored
+// (sample k's corners are read again), one past the hit or in a brick without
+// hits changes nothing.  A ray that grazes a surface jumps a hundred times, a
+// brick at a time, and the last warps of a launch wait for such rays alone:
+// the jump loop is one short dependent chain, without conversions between
+// integers and floats (which take ~20 cycles each) and without branches.
+// nsamp: samples evaluated, up to the hit; steps: jumps and evaluations; uniq
+// (DETAIL, one sample at a time): distinct corners of the samples evaluated.
+template <bool BF16, bool DETAIL, int PX, int NS = 3>
+__device__ __forceinline__ MarchHit march(const KParams& P, const MapPlanes& M, const Ray& r, bool active, float k0,
+                                          int& nsamp, int& steps, unsigned int& uniq) {
+    const uint32_t px = PX > 0 ? (uint32_t)PX : P.px;
+    const uint32_t pxy = PX > 0 ? (uint32_t)(PX * PX) : P.pxy;
+    const float hx = (float)P.nx - 0.5f, hy = (float)P.ny - 0.5f, hz = (float)P.nz - 0.5f;
+    const float rgx = r.rgx, rgy = r.rgy, rgz = r.rgz, cgx = r.cgx, cgy = r.cgy, cgz = r.cgz;
+    const float kmax = (float)P.kmax;
+    // k_safe: every sample k <= k_safe stays one voxel inside the grid
+    float k_safe = 0.0f;
+    if (cgx >= 0.5f && cgx <= hx - 1.0f && cgy >= 0.5f && cgy <= hy - 1.0f && cgz >= 0.5f && cgz <= hz - 1.0f) {
+        float ks = kmax;
+        const float rg3[3] = {rgx, rgy, rgz}, cg3[3] = {cgx, cgy, cgz}, h3[3] = {hx, hy, hz};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (rg3[a] > 0.0f) ks = fminf(ks, (h3[a] - 1.0f - cg3[a]) / (rg3[a] * P.eps32));
+            else if (rg3[a] < 0.0f) ks = fminf(ks, (0.5f - cg3[a]) / (rg3[a] * P.eps32));
+        }
+        k_safe = ks > 0.0f ? floorf(ks) : 0.0f;
+    }
+    const float ieps = 1.0f / P.eps32;
+    const ExitAxis ax(rgx, cgx, ieps), ay(rgy, cgy, ieps), az(rgz, cgz, ieps);
+    const bool skip = P.skip && M.boxes != nullptr;
+    MarchHit h;
+    h.k = 0;
+    h.f = h.f_prev = 0.0f;
+    h.prev_ok = false;
+    float k = k0;
+    float pfx = -2.0f, pfy = -2.0f, pfz = -2.0f;
+    bool fresh = true;   // DETAIL: the next evaluated sample starts a new run of corners
+    // sample k's position; false if the ray has ended
+    float gx, gy, gz;
+    auto position = [&](float kk) {
+        const float d = __fmul_rn(kk, P.eps32);
+        gx = __fmaf_rn(d, rgx, cgx);
+        gy = __fmaf_rn(d, rgy, cgy);
+        gz = __fmaf_rn(d, rgz, cgz);
+        return kk <= k_safe || (kk <= kmax && gx >= -0.5f && gx < hx && gy >= -0.5f && gy < hy && gz >= -0.5f && gz < hz);
+    };
+    bool live = active;
+    while (__any_sync(0xffffffffu, live)) {
+        const float k_in = k;
+        bool found = false;
+        while (live && !found) {
+            live = position(k);
+            ++steps;
+            uint32_t w = 0xffu, brick = 0u, cx = 0u, cy = 0u, cz = 0u;
+            if (skip && live) {
+                // cell coordinates, at least 0, + kFloorMagicBits, whose low 22 bits are 0
+                cx = max(__float_as_uint(__fadd_rd(gx, kFloorMagic)), kFloorMagicBits);
+                cy = max(__float_as_uint(__fadd_rd(gy, kFloorMagic)), kFloorMagicBits);
+                cz = max(__float_as_uint(__fadd_rd(gz, kFloorMagic)), kFloorMagicBits);
+                const int bi = box_index(P, (int)((cx >> 3) & 0x7ffffu), (int)((cy >> 3) & 0x7ffffu),
+                                         (int)((cz >> 3) & 0x7ffffu));
+                brick = ((cx >> 2) & 1u) | ((cy >> 1) & 2u) | (cz & 4u);
+                if (PRISM_IN_RANGE(P, CHK_RENDER_BRICK, bi, P.nbox)) w = __ldg(M.boxes + bi);
+            }
+            found = (w >> brick) & 1u;
+            const uint32_t c = (w >> 8) & 3u, clear = (4u << c) - 1u;   // an empty box of 4 2^c cells around it
+            const float ef = __uint_as_float((129u + c) << 23);
+            const float dm = fminf(fminf(ax.dist(cx, clear, ef), ay.dist(cy, clear, ef)), fminf(az.dist(cz, clear, ef), kmax));
+            // the first sample after the exit (dm < 2^22 but for enormous marches)
+            const float fl = P.kmax < (1 << 22) ? __fadd_rd(dm, kFloorMagic) - kFloorMagic : floorf(dm);
+            if (!found) k = fmaxf(fl, k) + 1.0f;
+        }
+        found = found && live;
+        if (k != k_in) {
+            h.prev_ok = false;
+            fresh = true;
+        }
+        __syncwarp();
+        if (found) {
+            ++nsamp;
+            position(k);
+            const Sample s0 = cell_of(px, pxy, gx, gy, gz);
+            if (!PRISM_IN_RANGE(P, CHK_RENDER_CORNER, (long long)s0.base + pxy + px + 1, P.npad)) {
+                live = false;
+            } else if constexpr (DETAIL) {
+                // consecutive cells share 8 >> (axes changed) corners (steps below one voxel)
+                const float flx = floorf(gx), fly = floorf(gy), flz = floorf(gz);
+                const int ch = (flx != pfx) + (fly != pfy) + (flz != pfz);
+                uniq += fresh ? 8u : 8u - (8u >> ch);
+                pfx = flx; pfy = fly; pfz = flz;
+                fresh = false;
+                h.f = trilinear<BF16, PX>(M.occ, s0.base, px, pxy, s0.fx, s0.fy, s0.fz);
+                if (h.f > P.tau32) {
+                    h.cur = s0;
+                    h.k = (int)k;
+                    live = false;
+                } else {
+                    h.f_prev = h.f;
+                    h.prev_ok = true;
+                    k += 1.0f;
+                }
+            } else {
+                // samples k .. k + NS - 1; one that the ray has not reads sample k's corners again
+                Sample sm[NS];
+                float f[NS];
+                bool ok[NS];
+                sm[0] = s0;
+                ok[0] = true;
+#pragma unroll
+                for (int j = 1; j < NS; ++j) {
+                    ok[j] = position(k + (float)j) && ok[j - 1];
+                    sm[j] = cell_of(px, pxy, gx, gy, gz);
+                    ok[j] = ok[j] && PRISM_IN_RANGE(P, CHK_RENDER_CORNER, (long long)sm[j].base + pxy + px + 1, P.npad);
+                    if (!ok[j]) sm[j] = s0;
+                }
+#pragma unroll
+                for (int j = 0; j < NS; ++j)
+                    f[j] = trilinear<BF16, PX>(M.occ, sm[j].base, px, pxy, sm[j].fx, sm[j].fy, sm[j].fz);
+                // the first one above tau, else the last one the ray has
+                bool hit = false;
+#pragma unroll
+                for (int j = 0; j < NS; ++j) {
+                    if (!hit && ok[j]) {
+                        hit = f[j] > P.tau32;
+                        if (j > 0) {
+                            ++nsamp;
+                            k += 1.0f;
+                            h.prev_ok = true;
+                            h.f_prev = f[j - 1];
+                        }
+                        if (hit) {
+                            h.cur = sm[j];
+                            h.f = f[j];
+                        }
+                        if (!hit && (j == NS - 1 || !ok[j + 1 < NS ? j + 1 : j])) h.f_prev = f[j];
+                    }
+                }
+                if (hit) {
+                    h.k = (int)k;
+                    live = false;
+                } else {
+                    h.prev_ok = true;
+                    k += 1.0f;
+                }
+            }
+        }
+    }
+    return h;
 }
 
 }  // namespace render_detail
 
 // One 16x8-pixel tile (128 threads; warp w covers the 8x4 pixels at
 // ((w & 1) 8, (w >> 1) 4) of the tile).  sR / sc: camera-to-world rotation
-// and centre in shared memory.  Returns the thread's march steps (jumps
-// and evaluating steps; 0 outside the image), the anchor render's tile cost.
-//
-// The march tests the grid bounds only for samples after k_safe, which a
-// conservative FP32 bound (one voxel of margin, far above the rounding of the
-// bound and of the sample positions) keeps inside the grid, and (with
-// P.skip) jumps over 4^3 bricks whose occupancy bound shows that no sample
-// in them can be a hit.  The samples evaluated, their corner indices and
-// the hit index are those of the one-loop march over every sample; the
-// value of a jumped-over sample k - 1 is recomputed at the hit.  With NS > 1
-// (not with DETAIL) the march evaluates NS consecutive samples per step, so
-// that a long ray has NS samples' loads in flight; it may also evaluate up
-// to NS - 1 samples past the hit, or inside a brick it would have jumped
-// from, none of which can change the hit (the first sample above tau) or
-// the outputs.  The sample count (DevStats::render_samples) leaves out
-// the samples evaluated past the hit.
-template <bool BF16, bool DETAIL, int PX, int NS = 1>
+// and centre in shared memory.  Returns the thread's march steps (0 outside
+// the image), the anchor render's tile cost.  The value of a sample k - 1
+// that the march did not evaluate is recomputed at the hit.
+template <bool BF16, bool DETAIL, int PX>
 __device__ __forceinline__ int render_tile(const KParams& P, const float* sR, const float* sc, const MapPlanes& M,
                                             float* __restrict__ depth, float* __restrict__ rgb,
                                             uint8_t* __restrict__ mask, int32_t* __restrict__ hitk,
@@ -214,172 +486,29 @@ __device__ __forceinline__ int render_tile(const KParams& P, const float* sR, co
     int nsamp = 0, hk = 0, steps = 0;
     unsigned int uniq = 0;   // distinct occupancy corners of this ray (DETAIL only)
     float out_d = 0.0f, out_r = 0.0f, out_g = 0.0f, out_b = 0.0f;
+    const render_detail::Ray r = render_detail::ray_of(P, sR, sc, u, v);
+    const float k0 = P.skip && M.boxes != nullptr
+                       ? render_detail::beam_start(P, M, sR, r, (float)(tile_x * 16 + (warp & 1) * 8) + 3.5f,
+                                                   (float)(tile_y * 8 + (warp >> 1) * 4) + 1.5f)
+                       : 1.0f;
+    const render_detail::MarchHit h = render_detail::march<BF16, DETAIL, PX>(P, M, r, active, k0, nsamp, steps, uniq);
     if (active) {
-        // ray set-up (FP32 recipe)
-        float dx = __fmul_rn(__fsub_rn((float)u, P.cx32), P.ifx32);
-        float dy = __fmul_rn(__fsub_rn((float)v, P.cy32), P.ify32);
-        float w0 = __fmaf_rn(sR[0], dx, __fmaf_rn(sR[1], dy, sR[2]));
-        float w1 = __fmaf_rn(sR[3], dx, __fmaf_rn(sR[4], dy, sR[5]));
-        float w2 = __fmaf_rn(sR[6], dx, __fmaf_rn(sR[7], dy, sR[8]));
-        float inv_n = __fdiv_rn(1.0f, __fsqrt_rn(__fmaf_rn(w0, w0, __fmaf_rn(w1, w1, __fmul_rn(w2, w2)))));
-        float rgx = __fmul_rn(__fmul_rn(w0, inv_n), P.inv_vs32);
-        float rgy = __fmul_rn(__fmul_rn(w1, inv_n), P.inv_vs32);
-        float rgz = __fmul_rn(__fmul_rn(w2, inv_n), P.inv_vs32);
-        float cgx = __fmaf_rn(__fsub_rn(sc[0], P.o32[0]), P.inv_vs32, -0.5f);
-        float cgy = __fmaf_rn(__fsub_rn(sc[1], P.o32[1]), P.inv_vs32, -0.5f);
-        float cgz = __fmaf_rn(__fsub_rn(sc[2], P.o32[2]), P.inv_vs32, -0.5f);
-        const float hx = (float)P.nx - 0.5f, hy = (float)P.ny - 0.5f, hz = (float)P.nz - 0.5f;
-
-        // k_safe: every sample k <= k_safe stays one voxel inside the grid
-        int k_safe = 0;
-        if (cgx >= 0.5f && cgx <= hx - 1.0f && cgy >= 0.5f && cgy <= hy - 1.0f && cgz >= 0.5f &&
-            cgz <= hz - 1.0f) {
-            float ks = (float)P.kmax;
-            const float rg3[3] = {rgx, rgy, rgz}, cg3[3] = {cgx, cgy, cgz}, h3[3] = {hx, hy, hz};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (rg3[a] > 0.0f) ks = fminf(ks, (h3[a] - 1.0f - cg3[a]) / (rg3[a] * P.eps32));
-                else if (rg3[a] < 0.0f) ks = fminf(ks, (0.5f - cg3[a]) / (rg3[a] * P.eps32));
-            }
-            k_safe = ks > 0.0f ? (int)ks : 0;
-            k_safe = k_safe < P.kmax ? k_safe : P.kmax;
-        }
-
-        float f = 0.0f, f_prev = 0.0f;
-        bool prev_ok = false;   // f_prev holds the value of sample k - 1
-        int k = 1;
-        float kf = 1.0f;        // (float)k, exact below 2^24
-        bool hit = false;
-        render_detail::Sample cur;
-        float pfx = -2.0f, pfy = -2.0f, pfz = -2.0f;
-        bool fresh = true;      // DETAIL: the next evaluated sample starts a new run of corners
-        int cur_brick = -1;
-        bool cur_skip = false;
-        const bool skip = P.skip && M.bb != nullptr;
-        // for the brick exits: 1 / rg (0 where rg = 0) and 1 / eps
-        const float irgx = rgx != 0.0f ? 1.0f / rgx : 0.0f, irgy = rgy != 0.0f ? 1.0f / rgy : 0.0f,
-                    irgz = rgz != 0.0f ? 1.0f / rgz : 0.0f, ieps = 1.0f / P.eps32;
-        while (k <= P.kmax) {
-            ++steps;
-            const float d = __fmul_rn(kf, P.eps32);
-            const float gx = __fmaf_rn(d, rgx, cgx), gy = __fmaf_rn(d, rgy, cgy), gz = __fmaf_rn(d, rgz, cgz);
-            if (k > k_safe && !(gx >= -0.5f && gx < hx && gy >= -0.5f && gy < hy && gz >= -0.5f && gz < hz)) break;
-            cur = render_detail::cell_of(px, pxy, gx, gy, gz);
-            if (skip) {
-                const int bx = max(cur.ix, 0) >> 2, by = max(cur.iy, 0) >> 2, bz = max(cur.iz, 0) >> 2;
-                const int brick = bx + 2 * P.nbx * (by + 2 * P.nby * bz);
-                if (brick != cur_brick) {
-                    cur_brick = brick;
-                    cur_skip = PRISM_IN_RANGE(P, CHK_RENDER_BRICK, brick, P.bb_len) &&
-                               render_detail::brick_skippable(P, M.bb, brick);
-                }
-                if (cur_skip) {   // no sample of this brick can be a hit: jump past it, or past
-                                  // the largest skippable brick above it (the bounds of the
-                                  // ancestors are loaded together, then the unbroken chain
-                                  // of skippable ones is climbed)
-                    bool up[3];
-#pragma unroll
-                    for (int l = 1; l <= 3; ++l) {
-                        up[l - 1] = false;
-                        if (l <= P.nlev) {
-                            const int dlx = (2 * P.nbx) >> l, dly = (2 * P.nby) >> l;
-                            const int qi = P.bb_off[l] + (bx >> l) + dlx * ((by >> l) + dly * (bz >> l));
-                            up[l - 1] = PRISM_IN_RANGE(P, CHK_RENDER_BRICK, qi, P.bb_len) &&
-                                        render_detail::brick_skippable(P, M.bb, qi);
-                        }
-                    }
-                    const int lv = up[0] ? (up[1] ? (up[2] ? 3 : 2) : 1) : 0;
-                    const int kn = render_detail::brick_exit(P, lv, bx >> lv, by >> lv, bz >> lv, irgx, irgy, irgz,
-                                                             cgx, cgy, cgz, ieps);
-                    k = kn > k ? kn : k + 1;
-                    kf = (float)k;
-                    prev_ok = false;
-                    fresh = true;
-                    continue;
-                }
-            }
-            ++nsamp;
-            if (DETAIL) {   // consecutive cells share 8 >> (axes changed) corners (steps below one voxel)
-                const float flx = floorf(gx), fly = floorf(gy), flz = floorf(gz);
-                const int ch = (flx != pfx) + (fly != pfy) + (flz != pfz);
-                uniq += fresh ? 8u : 8u - (8u >> ch);
-                pfx = flx; pfy = fly; pfz = flz;
-                fresh = false;
-            }
-            if (!PRISM_IN_RANGE(P, CHK_RENDER_CORNER, (long long)cur.base + pxy + px + 1, P.npad)) break;
-            if constexpr (NS > 1 && !DETAIL) {
-                // samples k .. k + NS - 1 together: their 8 NS corner loads are
-                // in flight at once.  A sample past kmax or leaving the grid
-                // ends the group (it re-reads sample k's corners, in bounds, and
-                // is ignored); one in a skippable brick is evaluated (its value
-                // cannot pass tau).  The first value above tau is the hit.
-                render_detail::Sample cs[NS];
-                bool ok[NS];
-                float fv[NS];
-                cs[0] = cur;
-                ok[0] = true;
-#pragma unroll
-                for (int j = 1; j < NS; ++j) {
-                    const float dj = __fmul_rn(kf + (float)j, P.eps32);
-                    const float jx = __fmaf_rn(dj, rgx, cgx), jy = __fmaf_rn(dj, rgy, cgy), jz = __fmaf_rn(dj, rgz, cgz);
-                    const render_detail::Sample sj = render_detail::cell_of(px, pxy, jx, jy, jz);
-                    ok[j] = ok[j - 1] && k + j <= P.kmax &&
-                            (k + j <= k_safe || (jx >= -0.5f && jx < hx && jy >= -0.5f && jy < hy && jz >= -0.5f && jz < hz)) &&
-                            PRISM_IN_RANGE(P, CHK_RENDER_CORNER, (long long)sj.base + pxy + px + 1, P.npad);
-                    cs[j] = cur;
-                    if (ok[j]) cs[j] = sj;
-                }
-#pragma unroll
-                for (int j = 0; j < NS; ++j)
-                    fv[j] = render_detail::trilinear<BF16, PX>(M.occ, cs[j].base, px, pxy, cs[j].fx, cs[j].fy, cs[j].fz);
-                int jh = -1, nv = 1;
-                float f_last = fv[0];
-#pragma unroll
-                for (int j = NS - 1; j >= 0; --j)
-                    if (ok[j] && fv[j] > P.tau32) jh = j;
-#pragma unroll
-                for (int j = 1; j < NS; ++j)
-                    if (ok[j]) { nv = j + 1; f_last = fv[j]; }
-                if (jh >= 0) {
-#pragma unroll
-                    for (int j = 0; j < NS; ++j)
-                        if (j == jh) {
-                            f = fv[j];
-                            if (j > 0) { f_prev = fv[j - 1]; prev_ok = true; cur = cs[j]; }
-                        }
-                    nsamp += jh;
-                    k += jh;
-                    hit = true;
-                    break;
-                }
-                nsamp += nv - 1;
-                f_prev = f_last;
-                prev_ok = true;
-                k += nv;
-                kf += (float)nv;
-                continue;
-            }
-            f = render_detail::trilinear<BF16, PX>(M.occ, cur.base, px, pxy, cur.fx, cur.fy, cur.fz);
-            if (f > P.tau32) { hit = true; break; }
-            f_prev = f;
-            prev_ok = true;
-            ++k;
-            kf += 1.0f;
-        }
-        if (hit && k == 1) hk = -1;
-        if (hit && k >= 2) {
+        const int k = h.k;
+        if (k == 1) hk = -1;
+        if (k >= 2) {
             hk = k;
+            const render_detail::Sample& cur = h.cur;
+            float f_prev = h.f_prev;
             // sample k - 1, recomputed exactly (same recipe) instead of carried along
             const float d1 = __fmul_rn((float)(k - 1), P.eps32);
-            const render_detail::Sample prev = render_detail::cell_of(px, pxy, __fmaf_rn(d1, rgx, cgx), __fmaf_rn(d1, rgy, cgy),
-                                        __fmaf_rn(d1, rgz, cgz));
+            const render_detail::Sample prev = render_detail::cell_of(px, pxy, __fmaf_rn(d1, r.rgx, r.cgx),
+                                        __fmaf_rn(d1, r.rgy, r.cgy), __fmaf_rn(d1, r.rgz, r.cgz));
             if (PRISM_IN_RANGE(P, CHK_RENDER_CORNER, (long long)prev.base + pxy + px + 1, P.npad)) {
-                // sample k - 1 was jumped over: its value, by the same recipe
-                if (!prev_ok) f_prev = render_detail::trilinear<BF16, PX>(M.occ, prev.base, px, pxy, prev.fx, prev.fy, prev.fz);
-                const float alpha = __fdiv_rn(P.tau32 - f_prev, f - f_prev);
+                if (!h.prev_ok) f_prev = render_detail::trilinear<BF16, PX>(M.occ, prev.base, px, pxy, prev.fx, prev.fy, prev.fz);
+                const float alpha = __fdiv_rn(P.tau32 - f_prev, h.f - f_prev);
                 const float dk = __fmul_rn((float)k, P.eps32);
                 const float dstar = fmaf(alpha, dk - d1, d1);
-                out_d = dstar * inv_n;
+                out_d = dstar * r.inv_n;
                 float a1 = render_detail::trilinear<BF16, PX>(M.r, cur.base, px, pxy, cur.fx, cur.fy, cur.fz);
                 float a0 = render_detail::trilinear<BF16, PX>(M.r, prev.base, px, pxy, prev.fx, prev.fy, prev.fz);
                 out_r = fmaf(alpha, a1 - a0, a0);
@@ -397,19 +526,22 @@ __device__ __forceinline__ int render_tile(const KParams& P, const float* sR, co
         if (mask) mask[p] = (uint8_t)(hk >= 2);
         if (hitk) hitk[p] = hk;
     }
-    if (stats) {
-        unsigned long long s = warp_sum_u64((unsigned long long)nsamp);
-        unsigned int hits = __popc(__ballot_sync(0xffffffffu, hk >= 2));
-        unsigned int rays = __popc(__ballot_sync(0xffffffffu, active));
-        if (DETAIL) {
-            const unsigned long long q = warp_sum_u64((unsigned long long)uniq);
-            if (lane == 0) atomicAdd(&stats->render_unique_corners, q);
-        }
+    if (stats) {   // one atomic a counter and block (four a block kept one L2 slice 40 % busy)
+        __shared__ unsigned long long s_stat[4][4];
+        const unsigned long long s = warp_sum_u64((unsigned long long)nsamp);
+        const unsigned long long q = DETAIL ? warp_sum_u64((unsigned long long)uniq) : 0ull;
+        const unsigned int hits = __popc(__ballot_sync(0xffffffffu, hk >= 2));
+        const unsigned int rays = __popc(__ballot_sync(0xffffffffu, active));
         if (lane == 0) {
-            atomicAdd(&stats->render_samples, s);
-            atomicAdd(&stats->render_hits, (unsigned long long)hits);
-            atomicAdd(&stats->render_rays, (unsigned long long)rays);
+            s_stat[warp][0] = rays;
+            s_stat[warp][1] = s;
+            s_stat[warp][2] = hits;
+            s_stat[warp][3] = q;
         }
+        __syncthreads();
+        if (threadIdx.x < (DETAIL ? 4 : 3))
+            atomicAdd(&stats->render_rays + threadIdx.x, s_stat[0][threadIdx.x] + s_stat[1][threadIdx.x] +
+                                                             s_stat[2][threadIdx.x] + s_stat[3][threadIdx.x]);
     }
     return steps;
 }

@@ -45,8 +45,8 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Byte layout of one stream's single device allocation.
 struct StreamLayout {
-    size_t plane, off_map, off_tb, off_bb, off_depth, off_rgb, off_omask, off_adepth, off_argb, off_a0, off_a1,
-        off_dev, off_stats, off_partials, off_counter, off_list, total;
+    size_t plane, off_map, off_bricks, off_boxes, off_depth, off_rgb, off_omask, off_adepth, off_argb, off_a0, off_a1,
+        off_dev, off_stats, off_partials, off_counter, off_list, off_clist, total;
     int max_blocks;
 };
 
@@ -66,10 +66,10 @@ StreamLayout layout_of(const prism_config* c, int storage, int sms) {
     auto take = [&](size_t bytes) { const size_t at = o; o += align256(bytes); return at; };
     L.plane = align256(npad * es);
     L.off_map = take(6 * L.plane);
-    L.off_tb = take((size_t)(c->nx / 4) * (c->ny / 4) * (c->nz / 4) * sizeof(float2));
     KParams kp;
     fill_kparams(c, kp);
-    L.off_bb = take((size_t)kp.bb_len * sizeof(float2));
+    L.off_bricks = take((size_t)kp.nbx * kp.nby * kp.nbz);
+    L.off_boxes = take((size_t)kp.nbox * sizeof(uint16_t));
     L.off_depth = take(npix * 4);
     L.off_rgb = take(npix * 12);
     L.off_omask = take(npix);
@@ -80,8 +80,9 @@ StreamLayout layout_of(const prism_config* c, int storage, int sms) {
     L.off_dev = take(sizeof(DevState));
     L.off_stats = take(sizeof(DevStats));
     L.off_partials = take((size_t)L.max_blocks * TRACK_NV_MAX * sizeof(float));
-    L.off_counter = take(2 * sizeof(unsigned int));
+    L.off_counter = take(3 * sizeof(unsigned int));
     L.off_list = take((size_t)kp.nbx * kp.nby * kp.nbz * sizeof(int));
+    L.off_clist = take((size_t)kp.nbx * kp.nby * kp.nbz * sizeof(int));
     L.total = o;
     return L;
 }
@@ -221,8 +222,8 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
     d.M.b = b + L.off_map + 3 * L.plane;
     d.M.var_occ = b + L.off_map + 4 * L.plane;
     d.M.var_rgb = b + L.off_map + 5 * L.plane;
-    d.M.tb = (float2*)(b + L.off_tb);
-    d.M.bb = (float2*)(b + L.off_bb);
+    d.M.bricks = (uint8_t*)(b + L.off_bricks);
+    d.M.boxes = (uint16_t*)(b + L.off_boxes);
     d.dev = (DevState*)(b + L.off_dev);
     d.stats = (DevStats*)(b + L.off_stats);
     d.depth = (float*)(b + L.off_depth);
@@ -236,6 +237,7 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
     d.counter = (unsigned int*)(b + L.off_counter);
     d.fuse_count = d.counter + 1;
     d.fuse_list = (int*)(b + L.off_list);
+    d.cells_list = (int*)(b + L.off_clist);
     d.pstride = L.max_blocks;
     d.grid_gn = track_launch_grid(st->kp, TRACK_GN, L.max_blocks);
     d.grid_lap = track_launch_grid(st->kp, TRACK_LAPLACE, L.max_blocks);
@@ -251,7 +253,7 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
             return e;
         *kernels += 1;
     }
-    if ((e = launch_tile_bounds(st->kp, d.M, S->stream)) != cudaSuccess) return e;
+    if ((e = launch_map_index(st->kp, d.M, S->stream)) != cudaSuccess) return e;
     *kernels += 2;
     *kernels += 1;
     // first state, as prism_set_state writes it (normalised pose, zero anchor)
@@ -270,7 +272,7 @@ cudaError_t setup_stream(prism_server* S, Stream* st, int slot, int* kernels) {
     // pageable source: the copy is staged before the call returns
     if ((e = cudaMemcpyAsync(d.dev, &ds, sizeof(ds), cudaMemcpyHostToDevice, S->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(d.stats, 0, sizeof(DevStats), S->stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(d.counter, 0, 2 * sizeof(unsigned int), S->stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(d.counter, 0, 3 * sizeof(unsigned int), S->stream)) != cudaSuccess) return e;
     PoseArg pa{};
     if ((e = launch_prep(d.dev, PREP_STATE, pa, S->stream)) != cudaSuccess) return e;
     *kernels += 1;
@@ -363,7 +365,7 @@ void run_batch(prism_server* S, std::unique_lock<std::mutex>& lk) {
         B.tiles_off[i + 1] = B.tiles_off[i] + d.tiles_x * ((st->kp.H + 7) / 8);
         B.pix_off[i + 1] = B.pix_off[i] + (npix + 255) / 256;
         B.cull_off[i + 1] = B.cull_off[i] + (st->kp.nbx * st->kp.nby * st->kp.nbz + 255) / 256;
-        B.brick_off[i + 1] = B.brick_off[i] + st->kp.bb_len - st->kp.bb_off[st->kp.nlev];
+        B.box_off[i + 1] = B.box_off[i] + st->kp.ntx * st->kp.nty * st->kp.ntz;
         ups.push_back({d.depth, d.rgb, q.depth, q.rgb, (size_t)npix});
         fl.ids[i] = id;
         fl.tags[i] = q.tag;

@@ -40,7 +40,8 @@ struct SlotDesc {
     float* partials;           // localisation partials, value-major with stride pstride
     unsigned int* counter;     // ticket of the localisation passes
     int* fuse_list;            // the tiles in this step's frustum (kb_cull)
-    unsigned int* fuse_count;  // how many; zero between batches
+    int* cells_list;           // the tiles whose cells may read one of their voxels
+    unsigned int* fuse_count;  // [2] how many of each; zero between batches
     int pstride;
     int grid_gn, grid_lap;     // virtual grids of the Gauss-Newton and Laplace passes
     int px_spec;               // render stride specialisation (render_px_specialisation)
@@ -64,7 +65,7 @@ struct BatchDesc {
     int tiles_off[kServeMaxSlots + 1];      // prefix sums over members: render tiles
     int pix_off[kServeMaxSlots + 1];        // 256-pixel blocks
     int cull_off[kServeMaxSlots + 1];       // 256-tile groups of 8^3 voxel tiles
-    int brick_off[kServeMaxSlots + 1];      // top-level bricks
+    int box_off[kServeMaxSlots + 1];        // 32^3 boxes
     int gn_off[kServeMaxSlots + 1];         // over localising members: Gauss-Newton virtual blocks
     int lap_off[kServeMaxSlots + 1];        // Laplace virtual blocks
     BatchMember m[kServeMaxSlots];
@@ -82,12 +83,12 @@ struct ServeOut {
 // Persistent grid sizes of the batched kernels (blocks), from the occupancy
 // calculator at server creation.
 struct BatchGrids {
-    int pix, track_gn, track_lap, fuse, render, bricks;
+    int pix, track_gn, track_lap, fuse, render, flags, codes;
 };
 
 cudaError_t batch_grids(bool bf16, BatchGrids* g);
 
-constexpr int kServeKernels = 9;   // of a batched step beside its n_gn Gauss-Newton passes
+constexpr int kServeKernels = 10;   // of a batched step beside its n_gn Gauss-Newton passes
 
 // Enqueues the batched step (kServeKernels + n_gn kernels) on s.
 cudaError_t launch_batch_step(const SlotDesc* slots, BatchDesc* batch, const double* imu, ServeOut* out, int n_gn,

@@ -112,49 +112,70 @@ __global__ void __launch_bounds__(256) kb_cull(const SlotDesc* __restrict__ slot
         __syncthreads();
         // a rejected localisation lists no tile: its frame is not fused
         cull_tiles(S.P, sM, sb, (item - b->cull_off[i]) * 256 + (int)threadIdx.x, S.dev->rejected != 0, S.fuse_list,
-                   S.fuse_count);
+                   S.P.skip ? S.cells_list : nullptr, S.fuse_count);
         __syncthreads();   // the shared matrices are reused by the next item
     }
 }
 
-// The map update of every member's listed tiles.  The members' item ranges
-// are the prefix sums of the counts kb_cull left on the device.
-template <bool BF16>
-__global__ void __launch_bounds__(256, 4) kb_fuse(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
-    pdl_enter();
-    __shared__ float sM[9], sb[3];
-    __shared__ int s_off[kServeMaxSlots + 1];
+// Item ranges of the members' lists (which = 0: fuse_list, 1: cells_list): the
+// prefix sums of the counts kb_cull left on the device.  Returns the total.
+__device__ __forceinline__ int list_offsets(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b, int which,
+                                            int* s_off) {
     const int n = b->n;
     if (threadIdx.x < kServeMaxSlots)
-        s_off[threadIdx.x + 1] = (int)threadIdx.x < n ? (int)*slots[b->m[threadIdx.x].slot].fuse_count : 0;
+        s_off[threadIdx.x + 1] = (int)threadIdx.x < n ? (int)slots[b->m[threadIdx.x].slot].fuse_count[which] : 0;
     __syncthreads();
     if (threadIdx.x == 0) {
         s_off[0] = 0;
         for (int i = 0; i < n; ++i) s_off[i + 1] += s_off[i];
     }
     __syncthreads();
-    const int total = s_off[n];
+    return s_off[n];
+}
+
+// The map update of every member's listed tiles.
+template <bool BF16>
+__global__ void __launch_bounds__(256, 4) kb_fuse(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
+    pdl_enter();
+    __shared__ float sM[9], sb[3];
+    __shared__ int s_off[kServeMaxSlots + 1];
+    const int n = b->n, total = list_offsets(slots, b, 0, s_off);
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int i = find_member(s_off, n, item);
         const SlotDesc& S = slots[b->m[i].slot];
         load_w2c(S.dev->w2c, sM, sb);
         __syncthreads();
         fuse_tile<BF16>(S.P, S.M, sM, sb, S.depth, S.rgb, S.o_mask, S.stats, (uint32_t)S.fuse_list[item - s_off[i]]);
-        __syncthreads();   // the shared matrices and reduction scratch are reused by the next item
+        __syncthreads();   // the shared matrices are reused by the next item
     }
 }
 
-// The brick bounds of every member after its fuse; item = one top-level
-// brick (render_dev.cuh).
-__global__ void __launch_bounds__(512) kb_bricks(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
+// The brick flags of every member's tiles that may read an updated voxel.
+template <bool BF16>
+__global__ void __launch_bounds__(256) kb_flags(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
     pdl_enter();
-    // the map update has read the frustum lists: their counts start the next batch at zero
-    if (blockIdx.x == 0 && (int)threadIdx.x < b->n) *slots[b->m[threadIdx.x].slot].fuse_count = 0u;
-    const int total = b->brick_off[b->n];
-    for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int i = find_member(b->brick_off, b->n, item);
+    __shared__ int s_off[kServeMaxSlots + 1];
+    const int n = b->n, total = list_offsets(slots, b, 1, s_off);
+    for (int item = 2 * blockIdx.x; item < total; item += 2 * gridDim.x) {
+        const int j = item + ((int)threadIdx.x >> 7), i = find_member(s_off, n, j < total ? j : item);
         const SlotDesc& S = slots[b->m[i].slot];
-        render_detail::brick_pyramid_block(S.P, S.M, item - b->brick_off[i]);
+        render_detail::brick_flags_tiles<BF16>(S.P, S.M, j < total ? S.cells_list[j - s_off[i]] : -1);
+    }
+}
+
+// The box codes of every member; item = one 32^3 box.
+__global__ void __launch_bounds__(256) kb_codes(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
+    pdl_enter();
+    // the lists have been read: their counts start the next batch at zero
+    if (blockIdx.x == 0 && (int)threadIdx.x < b->n) {
+        unsigned int* c = slots[b->m[threadIdx.x].slot].fuse_count;
+        c[0] = c[1] = 0u;
+    }
+    const int total = b->box_off[b->n];
+    for (int item = blockIdx.x; item < total; item += gridDim.x) {
+        const int i = find_member(b->box_off, b->n, item);
+        const SlotDesc& S = slots[b->m[i].slot];
+        render_detail::box_codes_block(S.P, S.M, item - b->box_off[i]);
     }
 }
 
@@ -227,7 +248,8 @@ int grid_of(K kern, int threads) {
 
 cudaError_t batch_grids(bool bf16, BatchGrids* g) {
     g->pix = grid_of(kb_mask, 256);
-    g->bricks = grid_of(kb_bricks, 512);
+    g->codes = grid_of(kb_codes, 256);
+    g->flags = bf16 ? grid_of(kb_flags<true>, 256) : grid_of(kb_flags<false>, 256);
     g->track_gn = grid_of(kb_track<TRACK_GN>, Block<TRACK_GN>::threads);
     g->track_lap = grid_of(kb_track<TRACK_LAPLACE>, Block<TRACK_LAPLACE>::threads);
     g->fuse = bf16 ? grid_of(kb_fuse<true>, 256) : grid_of(kb_fuse<false>, 256);
@@ -249,7 +271,9 @@ cudaError_t launch_batch_step(const SlotDesc* slots, BatchDesc* batch, const dou
     PRISM_BK(launch_pdl(kb_cull, g.pix, 256, s, slots, batch));
     if (bf16) PRISM_BK(launch_pdl(kb_fuse<true>, g.fuse, 256, s, slots, batch));
     else PRISM_BK(launch_pdl(kb_fuse<false>, g.fuse, 256, s, slots, batch));
-    PRISM_BK(launch_pdl(kb_bricks, g.bricks, 512, s, slots, batch));
+    if (bf16) PRISM_BK(launch_pdl(kb_flags<true>, g.flags, 256, s, slots, batch));
+    else PRISM_BK(launch_pdl(kb_flags<false>, g.flags, 256, s, slots, batch));
+    PRISM_BK(launch_pdl(kb_codes, g.codes, 256, s, slots, batch));
     if (bf16) PRISM_BK(launch_pdl(kb_render<true>, g.render, 128, s, slots, batch, n_gn + 1));
     else PRISM_BK(launch_pdl(kb_render<false>, g.render, 128, s, slots, batch, n_gn + 1));
     PRISM_BK(launch_pdl(kb_pack, g.pix, 256, s, slots, batch));
