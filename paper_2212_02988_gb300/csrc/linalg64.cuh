@@ -65,12 +65,32 @@ __device__ __forceinline__ double skew2_entry(const double w[3], double th2, int
 
 // Entry (i, j) of Exp(w) = I + a K + b K^2 (exp = true) or of J_l(w) =
 // I + b K + c K^2 (exp = false), K = [w]_x: one branch-free expression, so
-// that the lanes of a warp can evaluate entries of both.
+// that the lanes of a warp can evaluate entries of both.  Below 1/4 the two
+// coefficients come from two series with their constants selected by lane (the
+// operations of so3_coeffs, two of its three).
 __device__ __forceinline__ double so3_exp_jl_entry(const double w[3], bool exp, int i, int j) {
-    double a, b, c;
     const double th2 = fdot3(w[0], w[0], w[1], w[1], w[2], w[2]);
-    so3_coeffs(th2, a, b, c);
-    const double s1 = exp ? a : b, s2 = exp ? b : c;
+    double s1, s2;
+    if (th2 < 0.0625) {
+        const double x = th2;
+        s1 = fma(x, fma(x, fma(x, fma(x, fma(x, exp ? -1.0 / 39916800 : -1.0 / 479001600,
+                                             exp ? 1.0 / 362880 : 1.0 / 3628800),
+                                      exp ? -1.0 / 5040 : -1.0 / 40320),
+                               exp ? 1.0 / 120 : 1.0 / 720),
+                        exp ? -1.0 / 6 : -1.0 / 24),
+                 exp ? 1.0 : 0.5);
+        s2 = fma(x, fma(x, fma(x, fma(x, fma(x, exp ? -1.0 / 479001600 : -1.0 / 6227020800.0,
+                                             exp ? 1.0 / 3628800 : 1.0 / 39916800),
+                                      exp ? -1.0 / 40320 : -1.0 / 362880),
+                               exp ? 1.0 / 720 : 1.0 / 5040),
+                        exp ? -1.0 / 24 : -1.0 / 120),
+                 exp ? 0.5 : 1.0 / 6);
+    } else {
+        double a, b, c;
+        so3_coeffs(th2, a, b, c);
+        s1 = exp ? a : b;
+        s2 = exp ? b : c;
+    }
     return fma(s1, skew_entry(w, i, j), fma(s2, skew2_entry(w, th2, i, j), i == j ? 1.0 : 0.0));
 }
 
@@ -311,26 +331,27 @@ __device__ __forceinline__ double warp_ldlt6_solve(double a, bool* pd) {
         lm = 6;
     }
     bool ok = true;
-    double rown = 0.0;   // 1 / d_li, for this lane's row
+    double rsel = 0.0;   // 1 / d of this lane's column (a factor entry) or row (the right-hand side)
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         const double d = __shfl_sync(0xffffffffu, a, tri6(j, j));
         ok = ok && pivot_ok(d);
         const double rj = rcp64(d);
-        rown = sel64(li == j, rj, rown);
+        rsel = sel64(j == (rhs ? li : lm), rj, rsel);
         const bool below = li > j;                             // rows that column j updates
         const double aij = __shfl_sync(0xffffffffu, a, below ? tri6(li, j) : 0);
         const int src_m = lm == 6 ? 21 + j : (lm > j ? tri6(lm, j) : 0);
         const double amj = __shfl_sync(0xffffffffu, a, src_m);
-        const double lij = aij * rj;
         const double upd = fma(-(aij * amj), rj, a);
-        // the factor L_ij, kept for the back substitution; a trailing entry
-        // (lm <= li) or a right-hand side (lm = 6)
-        a = sel64(below && lm == j, lij, sel64(below && lm > j, upd, a));
+        // a trailing entry (lm <= li) or a right-hand side (lm = 6); column j
+        // itself keeps a_ij = L_ij d_j
+        a = sel64(below && lm > j, upd, a);
     }
+    // one product for all: the factor L_ij for the back substitution, and
     // z = D^-1 y on the right-hand-side lanes
-    double x = a * rown;
+    a = a * rsel;
+    double x = a;
     // back substitution: x_k is final once the rows below it are done
 #pragma unroll
     for (int k = 5; k >= 1; --k) {
@@ -343,14 +364,15 @@ __device__ __forceinline__ double warp_ldlt6_solve(double a, bool* pd) {
     return x;
 }
 
-// The inverse of a 6x6 symmetric positive definite A on one warp: the
+// The inverse of a 6x6 symmetric positive definite A on one warp, into out
+// (36 doubles, row-major, shared memory; the caller synchronises): the
 // factorisation A = L D L^T of warp_ldlt6_solve (lane e < 21 brings entry
 // (i, j), e = tri6(i, j), of A's lower triangle; the other lanes' values are
-// not used), then lane c < 6 solves L D L^T x = e_c (forward substitution,
-// D^-1, back substitution), so that x[0..5] of lane c is column c of A^-1
-// (other lanes: junk).  *pd: every pivot passed pivot_ok (every lane).  All
-// 32 lanes must call it.
-__device__ __forceinline__ void warp_spd6_inverse(double a, bool* pd, double x[6]) {
+// not used), then Y = L^-1 and A^-1 = Y^T D^-1 Y, one entry of the triangle a
+// lane: 4 and 5 steps of one FMA for all entries (a column a lane takes 15 and
+// 15, and an FP64 instruction ~64 cycles whatever lanes are active).  *pd:
+// every pivot passed pivot_ok (every lane).  All 32 lanes must call it.
+__device__ __forceinline__ void warp_spd6_inverse(double a, bool* pd, double* out) {
     const int lane = threadIdx.x & 31;
     const bool tri = lane < 21;
     int li = 5, lm = 6;
@@ -362,38 +384,45 @@ __device__ __forceinline__ void warp_spd6_inverse(double a, bool* pd, double x[6
         lm = lane - tri6(li, 0);
     }
     bool ok = true;
-    double r[6];
+    double rc = 0.0;   // 1 / d of this lane's column
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         const double d = __shfl_sync(0xffffffffu, a, tri6(j, j));
         ok = ok && pivot_ok(d);
-        r[j] = rcp64(d);
+        const double r = rcp64(d);
         const bool below = tri && li > j;
         const double aij = __shfl_sync(0xffffffffu, a, below ? tri6(li, j) : 0);
         const double amj = __shfl_sync(0xffffffffu, a, below && lm > j ? tri6(lm, j) : 0);
-        const double lij = aij * r[j];
-        const double upd = fma(-(aij * amj), r[j], a);
-        a = sel64(below && lm == j, lij, sel64(below && lm > j, upd, a));
+        const double upd = fma(-(aij * amj), r, a);
+        rc = sel64(lm == j, r, rc);
+        a = sel64(below && lm > j, upd, a);   // (column j itself keeps a_ij = L_ij d_j)
     }
-    // column c = lane of A^-1; L_ik (i > k) is in lane tri6(i, k)
-    const int c = lane < 6 ? lane : 0;
-    double y[6];
+    const double L = a * rc;               // strictly below the diagonal
+    const bool strict = tri && li > lm;
+    double y = -L;                         // Y_im: -(L_im + sum over m < k < i of L_ik Y_km)
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        double s = sel64(i == c, 1.0, 0.0);
-#pragma unroll
-        for (int k = 0; k < i; ++k) s = fma(-__shfl_sync(0xffffffffu, a, tri6(i, k)), y[k], s);
-        y[i] = s;
+    for (int k = 1; k < 5; ++k) {
+        const bool on = strict && k > lm && k < li;
+        const double lik = __shfl_sync(0xffffffffu, L, on ? tri6(li, k) : 0);
+        const double ykm = __shfl_sync(0xffffffffu, y, on ? tri6(k, lm) : 0);
+        y = sel64(on, fma(-lik, ykm, y), y);
     }
+    // (A^-1)_im = sum over k >= i of Y_ki Y_km / d_k (Y_ii = 1); z: Y_km / d_k of
+    // this lane's row, whose 1 / d_i the diagonal lane holds
+    const double ri = __shfl_sync(0xffffffffu, rc, tri ? tri6(li, li) : 0);
+    const double z = strict ? y * ri : ri;
+    double s = z;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) y[i] *= r[i];
-#pragma unroll
-    for (int i = 5; i >= 0; --i) {
-        double s = y[i];
-#pragma unroll
-        for (int k = i + 1; k < 6; ++k) s = fma(-__shfl_sync(0xffffffffu, a, tri6(k, i)), x[k], s);
-        x[i] = s;
+    for (int k = 1; k < 6; ++k) {
+        const bool on = tri && k > li;
+        const double yki = __shfl_sync(0xffffffffu, y, on ? tri6(k, li) : 0);
+        const double zkm = __shfl_sync(0xffffffffu, z, on ? tri6(k, lm) : 0);
+        s = sel64(on, fma(yki, zkm, s), s);
+    }
+    if (tri) {
+        out[6 * li + lm] = s;
+        out[6 * lm + li] = s;
     }
     *pd = ok;
 }
@@ -461,106 +490,6 @@ __device__ __forceinline__ void warp_gn_prior_terms(const double* Ra, const doub
         lp[e] = fdot3(Cb[ii], T[6 * (3 * bi) + j], Cb[3 + ii], T[6 * (3 * bi + 1) + j], Cb[6 + ii],
                       T[6 * (3 * bi + 2) + j]);
     }
-}
-
-// Block-cooperative inverse of an N x N SPD matrix (A and Ainv in shared
-// or global memory): warp 0 factors it (lane i holding row i) into the
-// shared scratch L / rdiag, then thread j solves for column j (unrolled);
-// the result is symmetrised.  Every thread of the block must call it.  Returns false (on
-// every thread) if not PD.
-template <int N>
-__device__ inline bool spd_inverse_block(const double* A, double* Ainv, double* L, double* rdiag, int* ok) {
-    static_assert(N <= 32, "one row a lane");
-    if (threadIdx.x < 32) {
-        // right-looking Cholesky on warp 0, lane i holding row i: each step is
-        // one warp instruction for all rows (GB300's FP64 pipe is paced by
-        // warp instructions, not lanes)
-        const int lane = threadIdx.x, row = lane < N ? lane : N - 1;
-        double a[N], r[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) a[j] = A[row * N + j];
-        bool pd = true;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const double d = __shfl_sync(0xffffffffu, a[j], j);
-            pd = pd && d > 0.0 && isfinite(d);
-            const double rj = rsqrt(d);
-            r[j] = rj;
-            if (lane > j) a[j] = a[j] * rj;   // L_ij
-#pragma unroll
-            for (int m = j + 1; m < N; ++m) {
-                const double lmj = __shfl_sync(0xffffffffu, a[j], m);
-                if (lane >= m) a[m] = fma(-a[j], lmj, a[m]);
-            }
-        }
-        if (lane < N) {
-            rdiag[lane] = r[lane];
-#pragma unroll
-            for (int j = 0; j < N; ++j)
-                if (j < lane) L[lane * N + j] = a[j];
-        }
-        if (lane == 0) *ok = pd ? 1 : 0;
-    }
-    __syncthreads();
-    const bool good = *ok != 0;
-    if (good && threadIdx.x < N) {
-        const int c = threadIdx.x;
-        double y[N], x[N];
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            double s = i == c ? 1.0 : 0.0;
-#pragma unroll
-            for (int k = 0; k < i; ++k) s = fma(-L[i * N + k], y[k], s);
-            y[i] = s * rdiag[i];
-        }
-#pragma unroll
-        for (int i = N - 1; i >= 0; --i) {
-            double s = y[i];
-#pragma unroll
-            for (int k = i + 1; k < N; ++k) s = fma(-L[k * N + i], x[k], s);
-            x[i] = s * rdiag[i];
-        }
-#pragma unroll
-        for (int i = 0; i < N; ++i) Ainv[i * N + c] = x[i];
-    }
-    __syncthreads();
-    if (good)
-        for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-            const int i = e / N, j = e % N;
-            if (i < j) {
-                const double m = 0.5 * (Ainv[i * N + j] + Ainv[j * N + i]);
-                Ainv[i * N + j] = Ainv[j * N + i] = m;
-            }
-        }
-    __syncthreads();
-    return good;
-}
-
-// C = A (N x K) * B (K x M), computed by the threads of a block (element per
-// thread); operands in shared memory.
-template <int N, int K, int M>
-__device__ inline void block_matmul(const double* A, const double* B, double* C) {
-    for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
-        const int i = e / M, j = e % M;
-        double s = 0.0;
-#pragma unroll
-        for (int l = 0; l < K; ++l) s = fma(A[i * K + l], B[l * M + j], s);
-        C[e] = s;
-    }
-    __syncthreads();
-}
-
-// C = A (N x K) * B^T (B: M x K)
-template <int N, int K, int M>
-__device__ inline void block_matmul_nt(const double* A, const double* B, double* C) {
-    for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
-        const int i = e / M, j = e % M;
-        double s = 0.0;
-#pragma unroll
-        for (int l = 0; l < K; ++l) s = fma(A[i * K + l], B[j * K + l], s);
-        C[e] = s;
-    }
-    __syncthreads();
 }
 
 }  // namespace prism

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) k_rollout_states(KParams P, const DevStat
     __syncthreads();
     for (int i = 0; i < k; ++i) {
         const int f = seq * k + i;
-        predict_block(P, dev, imu + 7 * row0[f], counts[f], dts[f]);
+        predict_block<PREP_NONE>(P, dev, imu + 7 * row0[f], counts[f], dts[f]);
         __syncthreads();
         // the prior becomes the state, and the frame's record
         const double* pr = prior_of(dev);

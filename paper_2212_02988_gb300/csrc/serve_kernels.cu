@@ -46,12 +46,7 @@ __global__ void __launch_bounds__(256) kb_predict(const SlotDesc* __restrict__ s
     if (k >= b->n_loc) return;
     const BatchMember& m = b->m[b->loc[k]];
     const SlotDesc& S = slots[m.slot];
-    predict_block(S.P, S.dev, imu + 7 * m.imu_off, m.n_imu, m.dt);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        PoseArg pa{};
-        prep_mats_warp(S.dev, PREP_REL, pa);
-    }
+    predict_block<PREP_REL>(S.P, S.dev, imu + 7 * m.imu_off, m.n_imu, m.dt);
 }
 
 // Depth validity of the observed frames.

@@ -7,20 +7,15 @@ namespace prism {
 __global__ void __launch_bounds__(256) k_predict(KParams P, DevState* dev, const double* __restrict__ imu, int n,
                                                  double dt) {
     pdl_enter();
-    predict_block(P, dev, imu, n, dt);
+    predict_block<PREP_NONE>(P, dev, imu, n, dt);
 }
 
-// The prediction, then (warp 0) the Gauss-Newton start matrices of the new
-// prior against the state mean's camera.
+// The prediction and the Gauss-Newton start matrices of the new prior against
+// the state mean's camera.
 __global__ void __launch_bounds__(256) k_predict_prep(KParams P, DevState* dev, const double* __restrict__ imu,
                                                       int n, double dt) {
     pdl_enter();
-    predict_block(P, dev, imu, n, dt);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        PoseArg pa{};
-        prep_mats_warp(dev, PREP_REL_NEXT, pa);
-    }
+    predict_block<PREP_REL_NEXT>(P, dev, imu, n, dt);
 }
 
 __global__ void k_prep(DevState* dev, int kind, PoseArg pose) {

@@ -670,11 +670,7 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
         }
         const double a = fma(2.0, S[L::oHT + 5 * lm - lm * (lm - 1) / 2 + li], Lp[6 * li + lm]);
         bool pd;
-        double x[6];
-        warp_spd6_inverse(a, &pd, x);
-        if (lane < 6)
-#pragma unroll
-            for (int k = 0; k < 6; ++k) Sa[6 * k + lane] = x[k];
+        warp_spd6_inverse(a, &pd, Sa);
         if (lane == 0) s_ok = pd;
     } else if (warp == 1) {   // meanwhile: D' = D Mi (D' = D on the translation columns)
 #pragma unroll
