@@ -67,9 +67,9 @@ __device__ __forceinline__ double from_ordered(unsigned long long u) {
 // twelve in a row, one FMA a row of positions, none a row of velocities), the
 // independent chains (IMU statistics, quaternions and rotation, reciprocals,
 // noise terms, start matrices) run on warps of different sub-partitions, and
-// the window's sums share their shuffle trees.  35.5 us before, PREDFIGS with
-// dense 12x12 products, five shuffles a sum and one warp's Cholesky with
-// reciprocal square roots.  The skipped products are by zeros: a covariance
+// the window's sums share their shuffle trees: 22.7 us alone with cold caches, 17.4
+// a prediction in a rollout's chain (35.5 and 22.2 with dense 12x12 products,
+// five shuffles a sum and one warp's Cholesky with reciprocal square roots).  The skipped products are by zeros: a covariance
 // with an entry that is not finite, which they turned into NaN everywhere, is
 // marked instead (bad) and rejected as before.
 constexpr int PREP_NONE = -1;
