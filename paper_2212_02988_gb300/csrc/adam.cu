@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kAdamThreads, 1)
     __shared__ double s_xi[6], s_C[18], s_anchor[7], s_pq[4], s_pt[3], s_prec[36];
     __shared__ float swarp[kAdamThreads / 32][N];
     __shared__ unsigned long long s_c0;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     if (tid < 7) s_anchor[tid] = dev->anchor_pose[tid];
     else if (tid < 11) s_pq[tid - 7] = dev->pq[tid - 7];
     else if (tid < 14) s_pt[tid - 11] = dev->pt[tid - 11];

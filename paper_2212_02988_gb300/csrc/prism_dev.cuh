@@ -11,6 +11,8 @@
 
 #include <utility>
 
+#include "linalg64.cuh"
+
 namespace prism {
 
 // ------------------------------------------------ programmatic dependent launch
@@ -264,13 +266,13 @@ __device__ __forceinline__ double quat_R_entry_rn(double w, double x, double y, 
     const int sh = 2 * e;
     auto pick = [&](uint32_t tab) {
         const uint32_t k = (tab >> sh) & 3u;
-        return k == 0u ? w : (k == 1u ? x : (k == 2u ? y : z));
+        return sel64(k == 0u, w, sel64(k == 1u, x, sel64(k == 2u, y, z)));
     };
     const double p = __dmul_rn(pick(kA), pick(kB));
     const double r = __dmul_rn(pick(kC), pick(kD));
-    const double u = __dmul_rn(2.0, __dadd_rn(p, ((kNeg >> e) & 1u) ? -r : r));
+    const double u = __dmul_rn(2.0, __dadd_rn(p, sel64(((kNeg >> e) & 1u) != 0u, -r, r)));
     const double du = __dsub_rn(1.0, u);
-    return ((kDiag >> e) & 1u) ? du : u;
+    return sel64(((kDiag >> e) & 1u) != 0u, du, u);
 }
 
 // The FP32 camera-to-world, world-to-camera and pose-to-anchor matrices of
@@ -313,9 +315,9 @@ __device__ __forceinline__ void warp_mats_rel(const double* pose, const double* 
     const double r0 = __shfl_sync(0xffffffffu, Re, j), r1 = __shfl_sync(0xffffffffu, Re, 3 + j),
                  r2 = __shfl_sync(0xffffffffu, Re, 6 + j);
     const bool mrow = e < 9;
-    const double b0 = mrow ? r0 : __dsub_rn(pose[0], anchor[0]);
-    const double b1 = mrow ? r1 : __dsub_rn(pose[1], anchor[1]);
-    const double b2 = mrow ? r2 : __dsub_rn(pose[2], anchor[2]);
+    const double b0 = sel64(mrow, r0, __dsub_rn(pose[0], anchor[0]));
+    const double b1 = sel64(mrow, r1, __dsub_rn(pose[1], anchor[1]));
+    const double b2 = sel64(mrow, r2, __dsub_rn(pose[2], anchor[2]));
     const double v = dot3_rn(a0, b0, a1, b1, a2, b2);
     if (lane < 12) out[lane] = (float)v;
 }

@@ -67,9 +67,12 @@ __device__ __forceinline__ double from_ordered(unsigned long long u) {
 // twelve in a row, one FMA a row of positions, none a row of velocities), the
 // independent chains (IMU statistics, quaternions and rotation, reciprocals,
 // noise terms, start matrices) run on warps of different sub-partitions, and
-// the window's sums share their shuffle trees: 22.7 us alone with cold caches, 17.4
-// a prediction in a rollout's chain (35.5 and 22.2 with dense 12x12 products,
-// five shuffles a sum and one warp's Cholesky with reciprocal square roots).  The skipped products are by zeros: a covariance
+// the window's sums share their shuffle trees: 11.4 us (35 with dense 12x12
+// products, five shuffles a sum and one warp's Cholesky with reciprocal square
+// roots).  The warp index is read from lane 0 so that the compiler knows the
+// branches on it to be warp-uniform: it otherwise takes every shuffle after
+// the first loop for a divergent one (~500 cycles each instead of 25; the
+// IMU statistics alone 16,800 cycles instead of 5,000).  The skipped products are by zeros: a covariance
 // with an entry that is not finite, which they turned into NaN everywhere, is
 // marked instead (bad) and rejected as before.
 constexpr int PREP_NONE = -1;
@@ -88,7 +91,7 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
     __shared__ double pose[7], anchor[7], Ra[9];
     __shared__ double Prec[36], Dm[36], W[36], LC[36];
     __shared__ int ok;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const double* state = reinterpret_cast<const double*>(reinterpret_cast<const char*>(dev) + offsetof(DevState, t));
     if (tid == 0) dev->flags = 0;   // a new step: only its own kernels raise flags
     bool bad = false;
@@ -98,24 +101,31 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
         const double inv_n = n > 0 ? 1.0 / n : 0.0;
         double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         unsigned long long te = ordered_bits(-1e300);
-        for (int i = lane; i < n; i += 32) {
-            for (int c = 0; c < 7; ++c) a[c] += imu[7 * i + c];
-            const unsigned long long k = ordered_bits(imu[7 * i]);
-            te = k > te ? k : te;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const bool in = i0 + lane < n;
+            const double* row = imu + 7 * (in ? i0 + lane : 0);
+            double x[7];
+            for (int c = 0; c < 7; ++c) x[c] = row[c];
+            for (int c = 0; c < 7; ++c) a[c] = sel64(in, a[c] + x[c], a[c]);
+            const unsigned long long k = ordered_bits(x[0]);
+            te = in && k > te ? k : te;
         }
         const double mean = warp_reduce_scatter64<8>(a) * inv_n;
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long k = __shfl_xor_sync(0xffffffffu, te, o);
             te = k > te ? k : te;
         }
-        if ((lane & 3) == 0) sums[lane >> 2] = lane == 28 ? from_ordered(te) : mean;
+        if ((lane & 3) == 0) sums[lane >> 2] = sel64(lane == 28, from_ordered(te), mean);
         __syncwarp();
         const double m0 = sums[0], m4[3] = {sums[4], sums[5], sums[6]};
         double f[4] = {0, 0, 0, 0};
-        for (int i = lane; i < n; i += 32) {
-            const double d = imu[7 * i] - m0;
-            f[0] = fma(d, d, f[0]);
-            for (int c = 0; c < 3; ++c) f[1 + c] = fma(d, imu[7 * i + 4 + c] - m4[c], f[1 + c]);
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const bool in = i0 + lane < n;
+            const double* row = imu + 7 * (in ? i0 + lane : 0);
+            const double d = row[0] - m0;
+            f[0] = sel64(in, fma(d, d, f[0]), f[0]);
+            for (int c = 0; c < 3; ++c) f[1 + c] = sel64(in, fma(d, row[4 + c] - m4[c], f[1 + c]), f[1 + c]);
         }
         const double fs = warp_reduce_scatter64<4>(f);
         if ((lane & 7) == 0) fit[lane >> 3] = fs;
@@ -124,7 +134,7 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
         quat_normalise(q);
         const double Re = quat_R_entry_rn(q[0], q[1], q[2], q[3], lane < 9 ? lane : 0);
         if (lane < 9) R0[lane] = Re;
-        else if (lane < 13) qm[lane - 9] = lane == 9 ? q[0] : (lane == 10 ? q[1] : (lane == 11 ? q[2] : q[3]));
+        else if (lane < 13) qm[lane - 9] = sel64(lane == 9, q[0], sel64(lane == 10, q[1], sel64(lane == 11, q[2], q[3])));
     } else {
         const int e = tid - 32;   // 0 .. 191
         if (e < 157) {
@@ -152,7 +162,7 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
             // Rh = Exp(dt wm / 2) entries on lanes 0..8, Rf = Exp(dt wm) on lanes 9..17
             const bool hf = lane < 9;
             const int e = lane < 9 ? lane : (lane < 18 ? lane - 9 : 0), ei = e / 3, ej = e % 3;
-            const double f = hf ? 0.5 * dt : dt;
+            const double f = sel64(hf, 0.5 * dt, dt);
             double vrot[3];
             for (int a = 0; a < 3; ++a) vrot[a] = f * __shfl_sync(0xffffffffu, wml, a);
             const double Ee = so3_exp_jl_entry(vrot, true, ei, ej);
@@ -185,8 +195,9 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
             const bool lin = lane < 3;
             const int rr = lane < 3 ? lane : (lane < 6 ? lane - 3 : 0);
             const double* M = Me + (lin ? 0 : 9) + 3 * rr;
-            const double y = fdot3(M[0], lin ? sums[1] : gend[0], M[1], lin ? sums[2] : gend[1], M[2], lin ? sums[3] : gend[2]);
-            const double ul = y + (lane == 2 ? -P.gravity : 0.0), ua = (y - X[10 + rr]) * inv_dt;
+            const double* v = lin ? sums + 1 : gend;
+            const double y = fdot3(M[0], v[0], M[1], v[1], M[2], v[2]);
+            const double ul = y + sel64(lane == 2, -P.gravity, 0.0), ua = (y - X[10 + rr]) * inv_dt;
             u = sel64(lin, ul, ua);
         }
         // the new velocities (lanes 0..5) and position (lanes 0..2)
@@ -207,7 +218,7 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
         // Rw = Exp(wdt) entries on lanes 0..8, J_l(wdt) dt on lanes 9..17
         const int e = lane < 9 ? lane : (lane < 18 ? lane - 9 : 0);
         const double v = so3_exp_jl_entry(wdt, lane < 9, e / 3, e % 3), vt = v * dt;
-        if (lane < 18) E[lane] = lane < 9 ? v : vt;
+        if (lane < 18) E[lane] = sel64(lane < 9, v, vt);
     }
     __syncthreads();
     // T1 = F C: rows 3..5 (rotation: Rw and Jd entries) on threads 0..35, rows
@@ -244,13 +255,13 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
         const double* jb = E + 9 + 3 * b;
         const bool pos = lane == 9, cross = lane >= 10 && lane < 19;
         const double q = qv[pos || lane == 19 ? 0 : 1];
-        const double x0 = (pos || lane == 19 ? dt : (cross ? E[lane - 1] : ja[0])) * q;
+        const double x0 = sel64(pos || lane == 19, dt, *(cross ? E + (lane - 1) : ja)) * q;
         const double x1 = ja[1] * q, x2 = ja[2] * q;
-        const double s0 = x0 * (pos ? dt : jb[0]);
+        const double s0 = x0 * sel64(pos, dt, jb[0]);
         const double s2 = fma(x2, jb[2], fma(x1, jb[1], s0));
         const double sp = P.sigma_pose[pos ? 0 : 1], qp = sp * sp;
         const double d = sel64(pos, s0, s2), dq = d + qp;
-        if (lane < 10) nz[lane] = pos || a == b ? dq : d;
+        if (lane < 10) nz[lane] = sel64(pos || a == b, dq, d);
         else if (lane < 20) nz[lane] = x0;
     } else if (tid >= 128 && tid < 200) {
         T1[72 + tid - 128] = Cv[72 + tid - 128];
@@ -265,31 +276,29 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
     // F C F^T + noise, into Cv: column j of T1 F^T as T1 above
     if (tid < 36) {
         const int i = tid / 3, a = tid % 3;
-        double add = 0.0;
-        if (i >= 3 && i < 6) add = nz[3 * (i - 3) + a];
-        else if (i >= 9) add = nz[10 + 3 * a + i - 9];
+        const double add = sel64(i >= 3 && i < 6, nz[i >= 3 && i < 6 ? 3 * (i - 3) + a : 0],
+                                 sel64(i >= 9, nz[i >= 9 ? 10 + 3 * a + i - 9 : 0], 0.0));
         Cv[12 * i + 3 + a] = f_row(T1 + 12 * i, 1, a) + add;
     } else if (warp == 2) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int e = lane + 32 * r, i = e < 36 ? e / 3 : 0, j = e % 3;
-            const double add = i == j ? nz[9] : (i == j + 6 ? nz[19] : 0.0);
+            const double add = sel64(i == j, nz[9], sel64(i == j + 6, nz[19], 0.0));
             const double s = fma(T1[12 * i + j + 6], dt, T1[12 * i + j]) + add;
             if (e < 36) Cv[12 * i + j] = s;
         }
     } else if (tid >= 128 && tid < 200) {
         const int i = (tid - 128) / 6, j = (tid - 128) % 6;
-        double add = 0.0;
-        if (i < 3) add = i == j ? nz[19] : 0.0;
-        else if (i < 6) add = j >= 3 ? nz[10 + 3 * (i - 3) + j - 3] : 0.0;
-        else if (i == j + 6) add = qv[j < 3 ? 0 : 1];
+        const bool rot = i >= 3 && i < 6 && j >= 3;
+        const double add = sel64(i < 3 && i == j, nz[19], sel64(rot, nz[rot ? 10 + 3 * (i - 3) + j - 3 : 0],
+                                                                sel64(i == j + 6, qv[j < 3 ? 0 : 1], 0.0)));
         Cv[12 * i + 6 + j] = T1[12 * i + 6 + j] + add;
     } else if (warp == 7 && PREP != PREP_NONE) {
         warp_mats_rel(pose, anchor, dev->rel);
     } else if (warp == 3 && PREP != PREP_NONE) {
         // the localisation's constants: q0 = conj(q_anchor) (x) q_prior, b0 = Ra^T (t_prior - t_anchor)
         const int c = lane & 3, i2 = lane < 3 ? lane : 0;
-        const double q0 = warp_quat_mul_component(c == 0 ? anchor[3] : -anchor[3 + c], pose + 3);
+        const double q0 = warp_quat_mul_component(sel64(c == 0, anchor[3], -anchor[3 + c]), pose + 3);
         const double b0 = fdot3(Ra[i2], pose[0] - anchor[0], Ra[3 + i2], pose[1] - anchor[1], Ra[6 + i2],
                                 pose[2] - anchor[2]);
         if (lane < 4) dev->gn_q0[lane] = q0;
@@ -298,8 +307,7 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
     __syncthreads();
     if (tid < 78) {   // the symmetric part, one entry of the lower triangle a thread
         const int i = (int)((sqrtf(8.0f * (float)tid + 1.0f) - 1.0f) * 0.5f), j = tid - i * (i + 1) / 2;
-        double m = 0.5 * (Cv[12 * i + j] + Cv[12 * j + i]);
-        if (bad) m = __longlong_as_double(0x7ff8000000000000ll);
+        const double m = sel64(bad, __longlong_as_double(0x7ff8000000000000ll), 0.5 * (Cv[12 * i + j] + Cv[12 * j + i]));
         Sig[12 * i + j] = m;
         Sig[12 * j + i] = m;
         dev->pcov[12 * i + j] = m;
@@ -405,7 +413,7 @@ __device__ __forceinline__ void prep_mats_warp(DevState* dev, int kind, const Po
             // the localisation's constants: q0 = conj(q_anchor) (x) q_prior on
             // lanes 24..27, b0 = Ra^T (t_prior - t_anchor) on lanes 28..30
             const int c = lane & 3;
-            const double q0 = warp_quat_mul_component(c == 0 ? qa[0] : -qa[c], dev->pq);
+            const double q0 = warp_quat_mul_component(sel64(c == 0, qa[0], -qa[c]), dev->pq);
             if (lane >= 24 && lane < 28) dev->gn_q0[c] = q0;
             const int i2 = lane >= 28 && lane < 31 ? lane - 28 : 0;
             const double rb0 = __shfl_sync(0xffffffffu, v, i2), rb1 = __shfl_sync(0xffffffffu, v, 3 + i2),

@@ -325,7 +325,9 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
     __shared__ int s_last, s_ok;
     __shared__ double st[kStage];
     __shared__ int s_nloc, s_flags;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (the warp index from lane 0: warp-uniform to the compiler, so that the
+    // finish's shuffles on one warp are not taken for divergent ones)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // Every block starts copying the state the last block's finish will need
     // (written by earlier kernels), so that it is in shared memory when the
     // last ticket is drawn.  (A cooperative launch's later passes find it,
