@@ -23,7 +23,7 @@ LIB_CHECKED = os.path.join(PKG, "libprism_checked.so")
 SOURCES = ["render.cu", "track.cu", "state.cu", "fuse.cu", "mapio.cu", "prism_abi.cu", "noalloc.cu",
            "render_bwd.cu", "serve_kernels.cu", "serve.cu", "adam.cu", "rollout.cu", "mapping.cu"]
 HEADERS = ["prism_dev.cuh", "linalg64.cuh", "kernels.h", "render_dev.cuh", "track_dev.cuh", "fuse_dev.cuh",
-           "state_dev.cuh", "serve.h", "host_util.h"]
+           "state_dev.cuh", "adjoint_dev.cuh", "serve.h", "host_util.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: device code contracts no multiply-add on its own, so every
 # value is the rounding sequence its source spells out (fused operations are
