@@ -178,16 +178,18 @@ cudaError_t launch_render_frames(const KParams& P, const float* mats, int frames
                                  float* rgb, int32_t* hitk, DevStats* stats, cudaStream_t s);
 
 // mapping.cu — gradient-descent mapping (the alternative to the closed-form
-// update).  launch_map_loss: over one rendered frame (depth, rgb, hit mask of
-// the render), where the render hit and obs_d is valid, the loss gradients
-// (d - D) / sd^2 and (c - C) / sc^2 replace depth and rgb (0 elsewhere) and
-// the loss terms are added to *loss.  launch_map_step: mu <- mu - lr (g +
-// (mu - mu0) / prior_var) on every padded element of the occupancy (g_occ, N
-// floats) and colour (g_rgb, 3N floats, linear layout) planes, the prior
-// term of the loss added to *loss; the empty-space index is left to the
-// caller.
-cudaError_t launch_map_loss(const KParams& P, float* depth, float* rgb, const uint8_t* mask, const float* obs_d,
-                            const float* obs_c, double sd, double sc, double* loss, cudaStream_t s);
+// update).  launch_descent_frames: up to kDescentBatch frames at known poses
+// (host, 7 doubles each, normalised; mats: 12 floats of scratch a frame): each is
+// rendered, and where the render hits and the observed depth is valid the loss
+// (d - D)^2 / (2 sd^2) + |c - C|^2 / (2 sc^2) is added to *loss and its gradient
+// through the render adjoint to g_occ (N floats) and g_rgb (3N floats, linear
+// layout).  launch_map_step: mu <- mu - lr (g + (mu - mu0) / prior_var) on every
+// padded element of the occupancy and colour planes, the prior term of the loss
+// added to *loss; the empty-space index is left to the caller.
+constexpr int kDescentBatch = 32;
+cudaError_t launch_descent_frames(const KParams& P, const double* poses, int frames, const MapPlanes& M,
+                                  const float* obs_d, const float* obs_c, double sd, double sc, float* mats,
+                                  float* g_occ, float* g_rgb, double* loss, DevStats* stats, bool detail, cudaStream_t s);
 cudaError_t launch_map_step(const KParams& P, const MapPlanes& M, const float* g_occ, const float* g_rgb,
                             double lr_occ, double lr_rgb, double mu0_occ, double mu0_rgb, double prior_var,
                             double* loss, cudaStream_t s);

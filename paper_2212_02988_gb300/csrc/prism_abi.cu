@@ -184,8 +184,8 @@ struct prism_ctx {
     char* h_roll = nullptr;
     size_t h_roll_cap = 0;
     cudaEvent_t ev_roll = nullptr;
-    // prism_map_descent's buffers: gradients (N + 3N floats), one rendered
-    // frame (depth, colour, hit mask) and the loss, in one block
+    // prism_map_descent's buffers: gradients (N + 3N floats), a batch of camera
+    // matrices and the loss, in one block
     void* md_dev = nullptr;
     // prism_step_host's device copies of the host frames, used in turn, and
     // the event after the last call's copies
@@ -1130,33 +1130,25 @@ prism_status prism_map_descent(prism_handle h, int32_t n, const double* poses, c
     const size_t npix = (size_t)h->cfg.width * h->cfg.height;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t o_grgb = up(h->nvox * sizeof(float));
-    const size_t o_rd = o_grgb + up(3 * h->nvox * sizeof(float));
-    const size_t o_rc = o_rd + up(npix * sizeof(float));
-    const size_t o_rm = o_rc + up(3 * npix * sizeof(float));
-    const size_t o_loss = o_rm + up(npix);
+    const size_t o_mats = o_grgb + up(3 * h->nvox * sizeof(float));
+    const size_t o_loss = o_mats + up(12 * kDescentBatch * sizeof(float));
     const size_t total = o_loss + 256;
     if (!h->md_dev) CK(h, dalloc(h, &h->md_dev, total), "descent buffers");
     char* b = (char*)h->md_dev;
     float* g_occ = (float*)b;
     float* g_rgb = (float*)(b + o_grgb);
-    float* r_d = (float*)(b + o_rd);
-    float* r_c = (float*)(b + o_rc);
-    uint8_t* r_m = (uint8_t*)(b + o_rm);
+    float* mats = (float*)(b + o_mats);
     double* d_loss = (double*)(b + o_loss);
-    CK(h, cudaMemsetAsync(g_occ, 0, o_rd, h->stream), "clear gradients");
+    CK(h, cudaMemsetAsync(g_occ, 0, o_mats, h->stream), "clear gradients");
     CK(h, cudaMemsetAsync(d_loss, 0, sizeof(double), h->stream), "clear loss");
-    for (int j = 0; j < n; ++j) {
-        PoseArg pa{};
-        normalise_pose(poses + 7 * j, pa.p);
-        LAUNCH(h, launch_prep(h->dstate, PREP_AUX_C2W, pa, h->stream), "pose matrices");
-        LAUNCH(h, launch_render(h->kp, h->dstate->aux, h->map, r_d, r_c, r_m, nullptr, h->dstats, nullptr, nullptr,
-                                h->detail, h->stream),
-               "render");
-        LAUNCH(h, launch_map_loss(h->kp, r_d, r_c, r_m, depth + npix * j, rgb + 3 * npix * j, sd, sc, d_loss,
-                                  h->stream),
-               "loss gradients");
-        LAUNCH(h, launch_render_bwd(h->kp, h->dstate->aux, h->map, r_d, r_c, g_occ, g_rgb, h->dstate, h->stream),
-               "render adjoint");
+    for (int j = 0; j < n; j += kDescentBatch) {
+        const int m = n - j < kDescentBatch ? n - j : kDescentBatch;
+        double p[7 * kDescentBatch];
+        for (int k = 0; k < m; ++k) normalise_pose(poses + 7 * (j + k), p + 7 * k);
+        LAUNCH(h, launch_descent_frames(h->kp, p, m, h->map, depth + npix * j, rgb + 3 * npix * j, sd, sc, mats, g_occ,
+                                        g_rgb, d_loss, h->dstats, h->detail, h->stream),
+               "descent frames");
+        ++h->launches;   // (two kernels: the matrices and the frames)
     }
     LAUNCH(h, launch_map_step(h->kp, h->map, g_occ, g_rgb, lr_occ, lr_rgb, h->cfg.init_occ, h->cfg.init_rgb,
                               h->cfg.prior_var, d_loss, h->stream),

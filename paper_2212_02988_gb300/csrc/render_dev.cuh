@@ -466,6 +466,28 @@ __device__ __forceinline__ MarchHit march(const KParams& P, const MapPlanes& M, 
 
 }  // namespace render_detail
 
+// The work counters of one 128-thread tile: one atomic a counter and block
+// (four a block kept one L2 slice 40 % busy).  Every thread calls it.
+template <bool DETAIL>
+__device__ __forceinline__ void tile_stats(DevStats* stats, bool active, bool hit, int nsamp, unsigned int uniq) {
+    __shared__ unsigned long long s_stat[4][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long s = warp_sum_u64((unsigned long long)nsamp);
+    const unsigned long long q = DETAIL ? warp_sum_u64((unsigned long long)uniq) : 0ull;
+    const unsigned int hits = __popc(__ballot_sync(0xffffffffu, hit));
+    const unsigned int rays = __popc(__ballot_sync(0xffffffffu, active));
+    if (lane == 0) {
+        s_stat[warp][0] = rays;
+        s_stat[warp][1] = s;
+        s_stat[warp][2] = hits;
+        s_stat[warp][3] = q;
+    }
+    __syncthreads();
+    if (threadIdx.x < (DETAIL ? 4 : 3))   // (the four counters are consecutive)
+        atomicAdd(&stats->render_rays + threadIdx.x, s_stat[0][threadIdx.x] + s_stat[1][threadIdx.x] +
+                                                         s_stat[2][threadIdx.x] + s_stat[3][threadIdx.x]);
+}
+
 // One 16x8-pixel tile (128 threads; warp w covers the 8x4 pixels at
 // ((w & 1) 8, (w >> 1) 4) of the tile).  sR / sc: camera-to-world rotation
 // and centre in shared memory.  Returns the thread's march steps (0 outside
@@ -526,23 +548,7 @@ __device__ __forceinline__ int render_tile(const KParams& P, const float* sR, co
         if (mask) mask[p] = (uint8_t)(hk >= 2);
         if (hitk) hitk[p] = hk;
     }
-    if (stats) {   // one atomic a counter and block (four a block kept one L2 slice 40 % busy)
-        __shared__ unsigned long long s_stat[4][4];
-        const unsigned long long s = warp_sum_u64((unsigned long long)nsamp);
-        const unsigned long long q = DETAIL ? warp_sum_u64((unsigned long long)uniq) : 0ull;
-        const unsigned int hits = __popc(__ballot_sync(0xffffffffu, hk >= 2));
-        const unsigned int rays = __popc(__ballot_sync(0xffffffffu, active));
-        if (lane == 0) {
-            s_stat[warp][0] = rays;
-            s_stat[warp][1] = s;
-            s_stat[warp][2] = hits;
-            s_stat[warp][3] = q;
-        }
-        __syncthreads();
-        if (threadIdx.x < (DETAIL ? 4 : 3))
-            atomicAdd(&stats->render_rays + threadIdx.x, s_stat[0][threadIdx.x] + s_stat[1][threadIdx.x] +
-                                                             s_stat[2][threadIdx.x] + s_stat[3][threadIdx.x]);
-    }
+    if (stats) tile_stats<DETAIL>(stats, active, hk >= 2, nsamp, uniq);
     return steps;
 }
 
