@@ -115,26 +115,31 @@ __device__ __forceinline__ int box_index(const KParams& P, int x, int y, int z) 
     return 64 * ((x >> 2) + P.ntx * ((y >> 2) + P.nty * (z >> 2))) + ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
 }
 
-// The flags of the 8 bricks of two 8^3 tiles (256 threads, 128 a tile; a
-// negative tile: none): a brick's cells read the 5^3 voxels from its lowest
+// The flags of the 8 bricks of 2 T 8^3 tiles (256 threads, T tiles for each 128;
+// a negative tile: none): a brick's cells read the 5^3 voxels from its lowest
 // one on, and it may hold a hit unless the largest of them is below tau as
 // above.  Warp w of a tile's four takes the layers z = 2 w .. 2 w + 2; its lane
-// l < 27 reads voxel x = l % 9 of the rows y = 3 i + l / 9: nine loads in flight
+// l < 27 reads voxel x = l % 9 of the rows y = 3 i + l / 9: 9 T loads in flight
 // a lane.  Latency bound: 4.2 us for 512 tiles, 8.8 us for the ~3,400 of a
-// 640x480 step, 36 us for the 32,768 of a 256^3 map (a tile a block through
-// shared memory: 4.3, 10.3 and 75 us; a tile a warp: 9.4, 10.8 and 43).
-template <bool BF16>
-__device__ __forceinline__ void brick_flags_tiles(const KParams& P, const MapPlanes& M, int tile) {
-    __shared__ float2 s_b[2][4][4];   // [tile][warp][brick x + 2 y]: largest value and magnitude
-    const int t = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
-    const bool on = tile >= 0 && PRISM_IN_RANGE(P, CHK_FUSE_TILE, tile, (long long)P.nbx * P.nby * P.nbz);
-    if (on) {
-        const int bx = tile % P.nbx, by = (tile / P.nbx) % P.nby, bz = tile / (P.nbx * P.nby);
-        const int l = lane < 27 ? lane : 26, x = l % 9, y0 = l / 9;
-        const uint32_t base = pad_index(P, 8 * bx + x, 8 * by + y0, 8 * bz + 2 * w);
-        float v[9];
+// 640x480 step, 36 us for the 32,768 of a 256^3 map (T = 1; a tile a block
+// through shared memory: 4.3, 10.3 and 75 us; a tile a warp: 9.4, 10.8 and 43).
+template <bool BF16, int T>
+__device__ __forceinline__ void brick_flags_tiles(const KParams& P, const MapPlanes& M, const int (&tile)[T]) {
+    __shared__ float2 s_b[2][T][4][4];   // [half][tile][warp][brick x + 2 y]: largest value and magnitude
+    const int half = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const int l = lane < 27 ? lane : 26, x = l % 9, y0 = l / 9;
+    float v[T][9];
+    bool on[T];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) v[i] = map_load_rw<BF16>(M.occ, base + P.px * (3u * (i % 3)) + P.pxy * (i / 3));
+    for (int t = 0; t < T; ++t) {
+        on[t] = tile[t] >= 0 && PRISM_IN_RANGE(P, CHK_FUSE_TILE, tile[t], (long long)P.nbx * P.nby * P.nbz);
+        const int q = on[t] ? tile[t] : 0, bx = q % P.nbx, by = (q / P.nbx) % P.nby, bz = q / (P.nbx * P.nby);
+        const uint32_t base = pad_index(P, 8 * bx + x, 8 * by + y0, 8 * bz + 2 * w);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) v[t][i] = map_load_rw<BF16>(M.occ, base + P.px * (3u * (i % 3)) + P.pxy * (i / 3));
+    }
+#pragma unroll
+    for (int t = 0; t < T; ++t)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {   // y: 0 .. 4 (rows 3 r + y0), then 4 .. 8
             float m = -INFINITY, a = 0.0f;
@@ -143,8 +148,8 @@ __device__ __forceinline__ void brick_flags_tiles(const KParams& P, const MapPla
                 const int r = i % 3;
                 if (r == (q == 0 ? 2 : 0)) continue;
                 const bool in = r != 1 || (q == 0 ? y0 <= 1 : y0 >= 1);
-                m = fmaxf(m, in ? v[i] : -INFINITY);
-                a = fmaxf(a, in ? fabsf(v[i]) : 0.0f);
+                m = fmaxf(m, in ? v[t][i] : -INFINITY);
+                a = fmaxf(a, in ? fabsf(v[t][i]) : 0.0f);
             }
             // over the lanes' rows (l, l + 9, l + 18), then x = 0 .. 4 into lane 0 and 4 .. 8 into lane 4
             auto reduce = [&](float z) {
@@ -156,15 +161,16 @@ __device__ __forceinline__ void brick_flags_tiles(const KParams& P, const MapPla
             };
             m = reduce(m);
             a = reduce(a);
-            if (lane == 0 || lane == 4) s_b[t][w][(lane >> 2) + 2 * q] = make_float2(m, a);
+            if (lane == 0 || lane == 4) s_b[half][t][w][(lane >> 2) + 2 * q] = make_float2(m, a);
         }
-    }
     __syncthreads();
-    if (w == 0 && on) {   // lane: brick x + 2 y + 4 z
-        const float2 b0 = s_b[t][2 * ((lane >> 2) & 1)][lane & 3], b1 = s_b[t][2 * ((lane >> 2) & 1) + 1][lane & 3];
-        const uint32_t f = __ballot_sync(0xffffffffu, !(fmaxf(b0.x, b1.x) < P.tau32 - 0x1p-18f * (1.0f + fmaxf(b0.y, b1.y))));
-        if (lane == 0) M.bricks[tile] = (uint8_t)(f & 0xffu);
-    }
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+        if (w == t) {   // lane: brick x + 2 y + 4 z
+            const float2 b0 = s_b[half][t][2 * ((lane >> 2) & 1)][lane & 3], b1 = s_b[half][t][2 * ((lane >> 2) & 1) + 1][lane & 3];
+            const uint32_t f = __ballot_sync(0xffffffffu, !(fmaxf(b0.x, b1.x) < P.tau32 - 0x1p-18f * (1.0f + fmaxf(b0.y, b1.y))));
+            if (lane == 0 && on[t]) M.bricks[tile[t]] = (uint8_t)(f & 0xffu);
+        }
     __syncthreads();   // s_b is reused by the next tiles
 }
 

@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(256) kb_flags(const SlotDesc* __restrict__ slo
     for (int item = 2 * blockIdx.x; item < total; item += 2 * gridDim.x) {
         const int j = item + ((int)threadIdx.x >> 7), i = find_member(s_off, n, j < total ? j : item);
         const SlotDesc& S = slots[b->m[i].slot];
-        render_detail::brick_flags_tiles<BF16>(S.P, S.M, j < total ? S.cells_list[j - s_off[i]] : -1);
+        const int tile[1] = {j < total ? S.cells_list[j - s_off[i]] : -1};
+        render_detail::brick_flags_tiles<BF16, 1>(S.P, S.M, tile);
     }
 }
 
