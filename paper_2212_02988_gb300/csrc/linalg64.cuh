@@ -492,4 +492,80 @@ __device__ __forceinline__ void warp_gn_prior_terms(const double* Ra, const doub
     }
 }
 
+// The same terms on two warps at once: warp_gn_prior_terms takes one warp
+// through both chains, 4,400 cycles, and the end of each Gauss-Newton pass
+// waited for it; the longer of these takes 2,900, as long as the next pass's
+// matrices beside it (localisation at 80x60 118.6 -> 113.5 us, at 640x480 123 ->
+// 121): _maps gives ci1, ji and L' (its lower triangle, mirrored),
+// _vector gives m.  The operations of each entry are those above.  scratch: 63
+// and 24 doubles.
+__device__ __forceinline__ void warp_gn_prior_maps(const double* Ra, const double* L, const double* xi, double* ci1,
+                                                   double* lp, double* ji, double* scratch) {
+    const int lane = threadIdx.x & 31;
+    double* Ji = scratch;         // J_l^-1 (9)
+    double* Ci = scratch + 9;     // diag blocks of Ci: Ra (9), J_l^-1 Ra (9)
+    double* T = scratch + 27;     // L Ci (36)
+    const int e9 = lane < 9 ? lane : 0, i9 = e9 / 3, j9 = e9 % 3;
+    const double v = so3_jl_inv_entry(xi + 3, i9, j9);
+    if (lane < 9) {
+        Ji[lane] = v;
+        ji[lane] = v;
+        Ci[lane] = Ra[lane];
+    }
+    __syncwarp();
+    const double c = fdot3(Ji[3 * i9], Ra[j9], Ji[3 * i9 + 1], Ra[3 + j9], Ji[3 * i9 + 2], Ra[6 + j9]);
+    if (lane < 9) {
+        Ci[9 + lane] = c;
+        ci1[lane] = c;
+    }
+    __syncwarp();
+    // T[k][j] = sum over the block of j: L[k][3 bj + l] Ci_bj[l][jj]
+#pragma unroll
+    for (int round = 0; round < 2; ++round) {
+        const int e = lane + 32 * round < 36 ? lane + 32 * round : 0, k = e / 6, j = e % 6, bj = j / 3, jj = j % 3;
+        const double* Cb = Ci + 9 * bj;
+        const double* Lk = L + 6 * k + 3 * bj;
+        const double t = fdot3(Lk[0], Cb[jj], Lk[1], Cb[3 + jj], Lk[2], Cb[6 + jj]);
+        if (lane + 32 * round < 36) T[e] = t;
+    }
+    __syncwarp();
+    // L' = Ci^T T: L'[i][j] = sum over the block of i: Ci_bi[k][ii] T[3 bi + k][j], i >= j
+    int i = 0;
+    if (lane < 21) {
+#pragma unroll
+        for (int r = 1; r < 6; ++r)
+            if (lane >= tri6(r, 0)) i = r;
+    }
+    const int j = lane < 21 ? lane - tri6(i, 0) : 0, bi = i / 3, ii = i % 3;
+    const double* Cb = Ci + 9 * bi;
+    const double q = fdot3(Cb[ii], T[6 * (3 * bi) + j], Cb[3 + ii], T[6 * (3 * bi + 1) + j], Cb[6 + ii],
+                           T[6 * (3 * bi + 2) + j]);
+    if (lane < 21) {
+        lp[6 * i + j] = q;
+        lp[6 * j + i] = q;
+    }
+}
+
+__device__ __forceinline__ void warp_gn_prior_vector(const double* Ra, const double* L, const double* xi, double* m,
+                                                     double* scratch) {
+    const int lane = threadIdx.x & 31;
+    double* Ji = scratch;         // J_l^-1 (9), then J_l^-1 Ra (9)
+    double* Lx = scratch + 18;    // L xi (6)
+    const int e9 = lane < 9 ? lane : 0, i9 = e9 / 3, j9 = e9 % 3, i6 = lane < 6 ? lane : 0;
+    const double v = so3_jl_inv_entry(xi + 3, i9, j9);
+    double lx = 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) lx = fma(L[6 * i6 + k], xi[k], lx);
+    if (lane < 9) Ji[lane] = v;
+    if (lane < 6) Lx[lane] = lx;
+    __syncwarp();
+    const double c = fdot3(Ji[3 * i9], Ra[j9], Ji[3 * i9 + 1], Ra[3 + j9], Ji[3 * i9 + 2], Ra[6 + j9]);
+    if (lane < 9) Ji[9 + lane] = c;
+    __syncwarp();
+    const int bi = i6 / 3, ii = i6 % 3;
+    const double* Cb = bi ? Ji + 9 : Ra;
+    const double r = fdot3(Cb[ii], Lx[3 * bi], Cb[3 + ii], Lx[3 * bi + 1], Cb[6 + ii], Lx[3 * bi + 2]);
+    if (lane < 6) m[lane] = r;
+}
+
 }  // namespace prism

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(Block<TRACK_GN>::threads, 1)
     pdl_enter();
     for (int pass = 0; pass < passes; ++pass)
         if (!track_item<TRACK_GN, false, true>(P, od, orgb, om, a0, a1, dev, partials, pstride, barrier, stats,
-                                               blockIdx.x, gridDim.x, nullptr, pass))
+                                               blockIdx.x, gridDim.x, nullptr, pass, pass == passes - 1))
             break;
 }
 

@@ -304,6 +304,8 @@ using namespace track_detail;
 // block holds the identical next iterate and its matrices in shared memory
 // and goes on to the next pass without a launch; block 0 also writes them
 // to the device state.  Partials alternate between two buffers by pass.
+// `last`: the launch's last pass (the FP64 pose of the iterate and the device
+// copy of its prior terms are needed only there).
 // Returns false when the launch's passes must stop (a system that is not
 // positive definite, or a barrier that timed out; both raise a flag).
 template <int MODE, bool MASKGEN = false, bool COOP = false>
@@ -312,7 +314,8 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
                                            const float4* __restrict__ a0, const float4* __restrict__ a1,
                                            DevState* dev, float* __restrict__ partials, int pstride,
                                            unsigned int* __restrict__ counter, DevStats* __restrict__ stats,
-                                           int vb, int nvb, uint8_t* __restrict__ om_out = nullptr, int pass = 0) {
+                                           int vb, int nvb, uint8_t* __restrict__ om_out = nullptr, int pass = 0,
+                                           bool last = true) {
     static_assert(!COOP || MODE == TRACK_GN, "the cooperative passes are Gauss-Newton passes");
     constexpr int N = NV<MODE>::value;
     constexpr int kThreads = Block<MODE>::threads, kWarps = Block<MODE>::warps;
@@ -604,6 +607,8 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
                 if (lane < 9) dev->rel[lane] = (float)me;
                 else if (tl) dev->rel[lane] = (float)be;
             }
+        } else if (warp == 1 && COOP && !last) {
+            if (lane < 6) st[36 + lane] = xn[lane];
         } else if (warp == 1) {   // the FP64 pose of the new iterate (the state mean after the last pass)
             const double qn = warp_quat_exp_mul_unit(xn + 3, st + 49);
             if (to_dev) {
@@ -614,19 +619,25 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
             if (COOP && lane < 6) st[36 + lane] = xn[lane];
         } else if (warp == 2) {   // meanwhile: the prior's anchor-frame terms of the new iterate
             if (!COOP) {
-                warp_gn_prior_terms(Ci, st, xn, dev->gn_Ci + 9, dev->gn_Lp, dev->gn_m, dev->gn_Ji, &sm[2][0]);
-            } else {   // into the staged slots (Ci's second block, L', m), J_l^-1 beside them
-                double* ji = &sm[5][0];   // (the scratch takes sm[2] and part of sm[3])
-                warp_gn_prior_terms(Ci, st, xn, st + 65, st + 74, st + 110, ji, &sm[2][0]);
+                warp_gn_prior_maps(Ci, st, xn, dev->gn_Ci + 9, dev->gn_Lp, dev->gn_Ji, &sm[2][0]);
+            } else {   // into the staged slots (Ci's second block, L'), J_l^-1 beside them
+                double* ji = &sm[5][0];   // (the scratch takes sm[2] and sm[3])
+                warp_gn_prior_maps(Ci, st, xn, st + 65, st + 74, ji, &sm[2][0]);
                 __syncwarp();
-                if (to_dev) {
-                    for (int e = lane; e < 60; e += 32) {
+                if (last && to_dev) {
+                    for (int e = lane; e < 54; e += 32) {
                         if (e < 9) dev->gn_Ci[9 + e] = st[65 + e];
                         else if (e < 45) dev->gn_Lp[e - 9] = st[74 + e - 9];
-                        else if (e < 51) dev->gn_m[e - 45] = st[110 + e - 45];
-                        else dev->gn_Ji[e - 51] = ji[e - 51];
+                        else dev->gn_Ji[e - 45] = ji[e - 45];
                     }
                 }
+            }
+        } else if (warp == 3) {
+            double* const m = COOP ? st + 110 : dev->gn_m;
+            warp_gn_prior_vector(Ci, st, xn, m, &sm[6][0]);
+            if (COOP && last && to_dev) {
+                __syncwarp();
+                if (lane < 6) dev->gn_m[lane] = st[110 + lane];
             }
         }
         if (COOP) __syncthreads();   // the next pass reads the new terms and matrices
