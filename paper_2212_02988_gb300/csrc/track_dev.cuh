@@ -170,29 +170,44 @@ struct TrackPix {
     bool ok;
 };
 
-// Decisions up to the anchor gathers of pixel p, and the gathers themselves,
-// issued together (nearest normal/depth and the four bilinear colour taps)
-// as soon as the projection is known.  ok = the pixel passed the mask,
-// z > 0 and both image-range tests; the remaining gates are in track_eval.
-// MASKGEN: the pixel's depth validity is evaluated here (depth_valid) and
-// stored to om_out instead of read from om.
-template <bool MASKGEN>
-__device__ __forceinline__ void track_fetch(const KParams& P, const float* sM, const float* sb,
-                                            const float* __restrict__ od, const float* __restrict__ orgb,
-                                            const uint8_t* __restrict__ om, uint8_t* __restrict__ om_out,
-                                            const float4* __restrict__ a0, const float4* __restrict__ a1, int p,
-                                            int W, float fW1, float fH1, float fW2, float fH2, TrackPix& q) {
+// An observed pixel: its validity, depth and colour.  MASKGEN: the depth
+// validity is evaluated here (depth_valid) and stored to om_out instead of
+// read from om.
+struct TrackObs {
     bool m;
+    float z, c0, c1, c2;
+};
+template <bool MASKGEN>
+__device__ __forceinline__ TrackObs track_observe(const KParams& P, const float* __restrict__ od,
+                                                  const float* __restrict__ orgb, const uint8_t* __restrict__ om,
+                                                  uint8_t* __restrict__ om_out, int p, int W) {
+    TrackObs o;
     if constexpr (MASKGEN) {
-        m = depth_valid(P, od, p % W, p / W);
-        om_out[p] = (uint8_t)m;
+        o.m = depth_valid(P, od, p % W, p / W);
+        om_out[p] = (uint8_t)o.m;
     } else {
-        m = om[p] != 0;
+        o.m = om[p] != 0;
     }
-    const float z = od[p];
-    q.c0 = orgb[3 * p];
-    q.c1 = orgb[3 * p + 1];
-    q.c2 = orgb[3 * p + 2];
+    o.z = od[p];
+    o.c0 = orgb[3 * p];
+    o.c1 = orgb[3 * p + 1];
+    o.c2 = orgb[3 * p + 2];
+    return o;
+}
+
+// Decisions up to the anchor gathers of an observed pixel p, and the gathers
+// themselves, issued together (nearest normal/depth and the four bilinear
+// colour taps) as soon as the projection is known.  ok = the pixel passed the
+// mask, z > 0 and both image-range tests; the remaining gates are in
+// track_eval.
+__device__ __forceinline__ void track_project(const KParams& P, const float* sM, const float* sb, const TrackObs& o,
+                                              const float4* __restrict__ a0, const float4* __restrict__ a1, int p,
+                                              int W, float fW1, float fH1, float fW2, float fH2, TrackPix& q) {
+    const bool m = o.m;
+    const float z = o.z;
+    q.c0 = o.c0;
+    q.c1 = o.c1;
+    q.c2 = o.c2;
     const int u = p % W, v = p / W;
     // ---- decisions (FP32 recipe) ----
     float Pc[3], X[3];
@@ -225,6 +240,16 @@ __device__ __forceinline__ void track_fetch(const KParams& P, const float* sM, c
         q.I01 = a1[b00 + W];
         q.I11 = a1[b00 + W + 1];
     }
+}
+
+template <bool MASKGEN>
+__device__ __forceinline__ void track_fetch(const KParams& P, const float* sM, const float* sb,
+                                            const float* __restrict__ od, const float* __restrict__ orgb,
+                                            const uint8_t* __restrict__ om, uint8_t* __restrict__ om_out,
+                                            const float4* __restrict__ a0, const float4* __restrict__ a1, int p,
+                                            int W, float fW1, float fH1, float fW2, float fH2, TrackPix& q) {
+    const TrackObs o = track_observe<MASKGEN>(P, od, orgb, om, om_out, p, W);
+    track_project(P, sM, sb, o, a0, a1, p, W, fW1, fH1, fW2, fH2, q);
 }
 
 // The remaining gates of a fetched pixel (valid anchor depth and colour taps,
@@ -283,6 +308,31 @@ __device__ __forceinline__ void track_eval(const KParams& P, const EvalConst& k,
         accumulate<MODE>(acc, J, rr[c], sw, k.ib_rgb, ar * k.ib_rgb);
     }
     acc[L::oCount] += 1.0f;
+}
+
+// The pose -> anchor matrices of an iterate xn, straight from it:
+// Ra^T Exp(xi_theta) R_prior = Exp(w) A0 with w = Ra^T xi_theta and
+// A0 = Ra^T R_prior = R(q0), so M = R(quat_exp(w) (x) q0) (unit to rounding) and
+// b = b0 + Ra^T xi_t.  One warp; me: M's entry `lane` on lanes 0..8, be: b's
+// entry lane - 9 on lanes 9..11.
+__device__ __forceinline__ void warp_iterate_mats(const double* Ra, const double* xn, const double* q0p,
+                                                  const double* b0, double& me, double& be) {
+    const int lane = threadIdx.x & 31;
+    // Lanes 0..2: w; lane 3: |xi_theta|^2; lanes 9..11: Ra^T xi_t.
+    const bool tl = lane >= 9 && lane < 12;
+    const int r = lane < 3 ? lane : (tl ? lane - 9 : 0);
+    const bool sq = lane == 3;
+    const double* v = tl ? xn : xn + 3;
+    const double d = fdot3(sq ? v[0] : Ra[r], v[0], sq ? v[1] : Ra[3 + r], v[1],
+                           sq ? v[2] : Ra[6 + r], v[2]);
+    const double w[3] = {__shfl_sync(0xffffffffu, d, 0), __shfl_sync(0xffffffffu, d, 1),
+                         __shfl_sync(0xffffffffu, d, 2)};
+    const double th2 = __shfl_sync(0xffffffffu, d, 3);
+    const double qr = warp_quat_mul_component(warp_quat_exp_component(w, th2), q0p);
+    const double q0 = __shfl_sync(0xffffffffu, qr, 0), q1 = __shfl_sync(0xffffffffu, qr, 1),
+                 q2 = __shfl_sync(0xffffffffu, qr, 2), q3 = __shfl_sync(0xffffffffu, qr, 3);
+    me = quat_R_entry_rn(q0, q1, q2, q3, lane < 9 ? lane : 0);
+    be = b0[r] + d;
 }
 
 }  // namespace track_detail
@@ -580,25 +630,10 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
         // block's shared copies, which block 0 also writes to the device
         const bool to_dev = !COOP || vb == 0;
         if (warp == 0) {
-            // The FP32 pose -> anchor matrices of the next pass, straight from
-            // xi (the critical path): Ra^T Exp(xi_theta) R_prior = Exp(w) A0 with
-            // w = Ra^T xi_theta and A0 = Ra^T R_prior = R(q0), so
-            // M = R(quat_exp(w) (x) q0) (unit to rounding) and b = b0 + Ra^T xi_t.
-            // Lanes 0..2: w; lane 3: |xi_theta|^2; lanes 9..11: Ra^T xi_t.
+            // The FP32 pose -> anchor matrices of the next pass (the critical path).
+            double me, be;
+            warp_iterate_mats(Ci, xn, st + 116, st + 120, me, be);
             const bool tl = lane >= 9 && lane < 12;
-            const int r = lane < 3 ? lane : (tl ? lane - 9 : 0);
-            const bool sq = lane == 3;
-            const double* v = tl ? xn : xn + 3;
-            const double d = fdot3(sq ? v[0] : Ci[r], v[0], sq ? v[1] : Ci[3 + r], v[1],
-                                   sq ? v[2] : Ci[6 + r], v[2]);
-            const double w[3] = {__shfl_sync(0xffffffffu, d, 0), __shfl_sync(0xffffffffu, d, 1),
-                                 __shfl_sync(0xffffffffu, d, 2)};
-            const double th2 = __shfl_sync(0xffffffffu, d, 3);
-            const double qr = warp_quat_mul_component(warp_quat_exp_component(w, th2), st + 116);
-            const double q0 = __shfl_sync(0xffffffffu, qr, 0), q1 = __shfl_sync(0xffffffffu, qr, 1),
-                         q2 = __shfl_sync(0xffffffffu, qr, 2), q3 = __shfl_sync(0xffffffffu, qr, 3);
-            const double me = quat_R_entry_rn(q0, q1, q2, q3, lane < 9 ? lane : 0);
-            const double be = st[120 + r] + d;
             if (COOP) {
                 if (lane < 9) sM[lane] = (float)me;
                 else if (tl) sb[lane - 9] = (float)be;
