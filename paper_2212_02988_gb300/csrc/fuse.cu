@@ -19,7 +19,9 @@ __global__ void __launch_bounds__(256) k_fuse_cull(KParams P, const float* __res
     cull_tiles(P, sM, sb, blockIdx.x * blockDim.x + threadIdx.x, rejected && *rejected, list, cells_list, ctr);
 }
 
-// Persistent over the listed tiles (ctr[0] of them).
+// Persistent over the listed tiles (ctr[0] of them); a block reads its next
+// tile of the list beside the current one.  Bound by the latency of three
+// dependent rounds of loads (pixel, update decision, colours) at half the warps.
 template <bool BF16>
 __global__ void __launch_bounds__(256, 4) k_fuse_list(KParams P, MapPlanes M, const float* __restrict__ w2c,
                                                    const float* __restrict__ depth, const float* __restrict__ rgb,
@@ -27,11 +29,19 @@ __global__ void __launch_bounds__(256, 4) k_fuse_list(KParams P, MapPlanes M, co
                                                    const int* __restrict__ list, const unsigned int* __restrict__ ctr) {
     pdl_enter();
     __shared__ float sM[9], sb[3];
+    __shared__ unsigned int s_count[2];
     load_w2c(w2c, sM, sb);
+    if (threadIdx.x < 2) s_count[threadIdx.x] = 0u;
     __syncthreads();
     const unsigned int count = ctr[0];
-    for (unsigned int i = blockIdx.x; i < count; i += gridDim.x)
-        fuse_tile<BF16>(P, M, sM, sb, depth, rgb, mask, stats, (uint32_t)list[i]);
+    int tile = blockIdx.x < count ? list[blockIdx.x] : 0;
+    for (unsigned int i = blockIdx.x; i < count; i += gridDim.x) {
+        const int cur = tile;
+        if (i + gridDim.x < count) tile = list[i + gridDim.x];
+        fuse_tile<BF16>(P, M, sM, sb, depth, rgb, mask, s_count, (uint32_t)cur);
+    }
+    __syncthreads();
+    add_fuse_counts(stats, s_count);
 }
 
 template <bool BF16>

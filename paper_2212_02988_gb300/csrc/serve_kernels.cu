@@ -134,15 +134,19 @@ __global__ void __launch_bounds__(256, 4) kb_fuse(const SlotDesc* __restrict__ s
     pdl_enter();
     __shared__ float sM[9], sb[3];
     __shared__ int s_off[kServeMaxSlots + 1];
+    __shared__ unsigned int s_count[kServeMaxSlots][2];   // update counts by member
+    if (threadIdx.x < 2 * kServeMaxSlots) s_count[threadIdx.x >> 1][threadIdx.x & 1] = 0u;
     const int n = b->n, total = list_offsets(slots, b, 0, s_off);
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int i = find_member(s_off, n, item);
         const SlotDesc& S = slots[b->m[i].slot];
         load_w2c(S.dev->w2c, sM, sb);
         __syncthreads();
-        fuse_tile<BF16>(S.P, S.M, sM, sb, S.depth, S.rgb, S.o_mask, S.stats, (uint32_t)S.fuse_list[item - s_off[i]]);
+        fuse_tile<BF16>(S.P, S.M, sM, sb, S.depth, S.rgb, S.o_mask, s_count[i], (uint32_t)S.fuse_list[item - s_off[i]]);
         __syncthreads();   // the shared matrices are reused by the next item
     }
+    __syncthreads();
+    for (int i = 0; i < n; ++i) add_fuse_counts(slots[b->m[i].slot].stats, s_count[i]);
 }
 
 // The brick flags of every member's tiles that may read an updated voxel.
