@@ -665,8 +665,7 @@ __device__ __forceinline__ void depth_mask_px(const KParams& P, const float* __r
 // n = normalize((P(u+1,v) - P(u-1,v)) x (P(u,v+1) - P(u,v-1))), facing the camera.
 // anchor_pack_core takes the pixel's depth dc and its neighbours' (dr: u + 1,
 // dl: u - 1, dd: v + 1, du: v - 1), its depth validity mc and ok = it and its
-// four neighbours are valid inside the image border; the two packers below
-// only differ in where those come from.
+// four neighbours are valid inside the image border.
 __device__ __forceinline__ void anchor_pack_core(const KParams& P, int u, int v, float dc, float dr, float dl,
                                                  float dd, float du, bool mc, bool ok,
                                                  const float* __restrict__ rgb, float4* __restrict__ a0,
@@ -698,27 +697,6 @@ __device__ __forceinline__ void anchor_pack_core(const KParams& P, int u, int v,
     if (!ok) n0 = n1 = n2 = 0.0f;
     a0[p] = make_float4(n0, n1, n2, ok ? dc : 0.0f);
     a1[p] = make_float4(rgb[3 * p], rgb[3 * p + 1], rgb[3 * p + 2], mc ? 1.0f : 0.0f);
-}
-
-// One pixel from global memory (the validity of the pixel and of its four
-// neighbours evaluated here by depth_valid).
-__device__ __forceinline__ void anchor_pack_px(const KParams& P, const float* __restrict__ depth,
-                                               const float* __restrict__ rgb, float4* __restrict__ a0,
-                                               float4* __restrict__ a1, int p) {
-    const int u = p % P.W, v = p / P.W, W = P.W;
-    const bool mc = depth_valid(P, depth, u, v);
-    const bool ok = u >= 1 && u <= P.W - 2 && v >= 1 && v <= P.H - 2 && mc && depth_valid(P, depth, u - 1, v) &&
-                    depth_valid(P, depth, u + 1, v) && depth_valid(P, depth, u, v - 1) &&
-                    depth_valid(P, depth, u, v + 1);
-    const float dc = depth[p];
-    float dr = 0.0f, dl = 0.0f, dd = 0.0f, du = 0.0f;
-    if (ok) {
-        dr = depth[p + 1];
-        dl = depth[p - 1];
-        dd = depth[p + W];
-        du = depth[p - W];
-    }
-    anchor_pack_core(P, u, v, dc, dr, dl, dd, du, mc, ok, rgb, a0, a1, p);
 }
 
 // One 32x8-pixel tile on a block of 256 threads: the depths of the tile and

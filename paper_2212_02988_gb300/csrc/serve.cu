@@ -364,6 +364,7 @@ void run_batch(prism_server* S, std::unique_lock<std::mutex>& lk) {
         const int npix = st->kp.W * st->kp.H;
         B.tiles_off[i + 1] = B.tiles_off[i] + d.tiles_x * ((st->kp.H + 7) / 8);
         B.pix_off[i + 1] = B.pix_off[i] + (npix + 255) / 256;
+        B.pack_off[i + 1] = B.pack_off[i] + pack_tiles(st->kp);
         B.cull_off[i + 1] = B.cull_off[i] + (st->kp.nbx * st->kp.nby * st->kp.nbz + 255) / 256;
         B.box_off[i + 1] = B.box_off[i] + st->kp.ntx * st->kp.nty * st->kp.ntz;
         ups.push_back({d.depth, d.rgb, q.depth, q.rgb, (size_t)npix});

@@ -64,6 +64,7 @@ struct BatchDesc {
     int loc[kServeMaxSlots];                // their member indices
     int tiles_off[kServeMaxSlots + 1];      // prefix sums over members: render tiles
     int pix_off[kServeMaxSlots + 1];        // 256-pixel blocks
+    int pack_off[kServeMaxSlots + 1];       // 32x8-pixel tiles of the anchor packing
     int cull_off[kServeMaxSlots + 1];       // 256-tile groups of 8^3 voxel tiles
     int box_off[kServeMaxSlots + 1];        // 32^3 boxes
     int gn_off[kServeMaxSlots + 1];         // over localising members: Gauss-Newton virtual blocks
@@ -83,10 +84,11 @@ struct ServeOut {
 // Persistent grid sizes of the batched kernels (blocks), from the occupancy
 // calculator at server creation.
 struct BatchGrids {
-    int pix, track_gn, track_lap, fuse, render, flags, codes;
+    int pix, pack, track_gn, track_lap, fuse, render, flags, codes;
 };
 
 cudaError_t batch_grids(bool bf16, BatchGrids* g);
+int pack_tiles(const KParams& P);   // anchor-packing items of a stream
 
 constexpr int kServeKernels = 10;   // of a batched step beside its n_gn Gauss-Newton passes
 

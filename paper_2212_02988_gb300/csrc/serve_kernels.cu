@@ -75,14 +75,18 @@ __global__ void __launch_bounds__(256) kb_mask(const SlotDesc* __restrict__ slot
     }
 }
 
+// The anchors' packing; item = one 32x8-pixel tile.  Pixel by pixel from global
+// memory, with the validity of five pixels tested anew at each, a batch of nine
+// streams of 160x120 to 640x480 took 45 us; by tiles 33 us.
 __global__ void __launch_bounds__(256) kb_pack(const SlotDesc* __restrict__ slots, const BatchDesc* __restrict__ b) {
     pdl_enter();
-    const int total = b->pix_off[b->n];
+    const int total = b->pack_off[b->n];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const int i = find_member(b->pix_off, b->n, item);
+        const int i = find_member(b->pack_off, b->n, item);
         const SlotDesc& S = slots[b->m[i].slot];
-        const int p = (item - b->pix_off[i]) * 256 + threadIdx.x;
-        if (p < S.P.W * S.P.H) anchor_pack_px(S.P, S.a_depth, S.a_rgb, S.a0, S.a1, p);
+        const int t = item - b->pack_off[i], across = (S.P.W + kPackTW - 1) / kPackTW;
+        anchor_pack_tile(S.P, S.a_depth, S.a_rgb, S.a0, S.a1, t % across, t / across);
+        __syncthreads();   // the tile's shared memory is reused by the next item
     }
 }
 
@@ -264,8 +268,11 @@ int grid_of(K kern, int threads) {
 
 }  // namespace
 
+int pack_tiles(const KParams& P) { return ((P.W + kPackTW - 1) / kPackTW) * ((P.H + kPackTH - 1) / kPackTH); }
+
 cudaError_t batch_grids(bool bf16, BatchGrids* g) {
     g->pix = grid_of(kb_mask, 256);
+    g->pack = grid_of(kb_pack, 256);
     g->codes = grid_of(kb_codes, 256);
     g->flags = bf16 ? grid_of(kb_flags<true>, 256) : grid_of(kb_flags<false>, 256);
     g->track_gn = grid_of(kb_track<TRACK_GN>, Block<TRACK_GN>::threads);
@@ -294,7 +301,7 @@ cudaError_t launch_batch_step(const SlotDesc* slots, BatchDesc* batch, const dou
     PRISM_BK(launch_pdl(kb_codes, g.codes, 256, s, slots, batch));
     if (bf16) PRISM_BK(launch_pdl(kb_render<true>, g.render, 128, s, slots, batch, n_gn + 1));
     else PRISM_BK(launch_pdl(kb_render<false>, g.render, 128, s, slots, batch, n_gn + 1));
-    PRISM_BK(launch_pdl(kb_pack, g.pix, 256, s, slots, batch));
+    PRISM_BK(launch_pdl(kb_pack, g.pack, 256, s, slots, batch));
     PRISM_BK(launch_pdl(kb_out, kServeMaxSlots, 256, s, slots, batch, out));
 #undef PRISM_BK
     return cudaSuccess;
