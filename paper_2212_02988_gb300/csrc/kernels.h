@@ -17,6 +17,12 @@ struct PoseArg {
     const double* dev;
 };
 
+// A state as the host gives it, in the order of DevState's head (quaternion normalised).
+struct StateArg {
+    double t[3], q[4], v[3], w[3], cov[144];
+    int n_localised;
+};
+
 // Which FP32 matrices k_prep derives from an FP64 pose.
 enum PrepKind : int {
     PREP_STATE = 0,   // c2w and w2c of the state mean
@@ -117,6 +123,7 @@ cudaError_t launch_adam(const KParams& P, const float* o_depth, const float* o_r
 cudaError_t launch_predict(const KParams& P, DevState* dev, const double* imu, int n, double dt,
                            cudaStream_t s, bool pdl = true);
 cudaError_t launch_prep(DevState* dev, int kind, const PoseArg& pose, cudaStream_t s, bool pdl = true);
+cudaError_t launch_set_state(DevState* dev, const StateArg& state, cudaStream_t s);
 // The prediction followed, in the same block, by the PREP_REL_NEXT matrices of
 // the prior's mean (a plain launch).
 cudaError_t launch_predict_prep(const KParams& P, DevState* dev, const double* imu, int n, double dt,

@@ -402,8 +402,7 @@ prism_status read_state(prism_handle h, prism_state* out) {
 }
 
 prism_status write_state(prism_handle h, const prism_state* s) {
-    DevState d;
-    std::memset(&d, 0, sizeof(d));
+    StateArg d;
     double pin[7], pn[7];
     std::memcpy(pin, s->t, 3 * sizeof(double));
     std::memcpy(pin + 3, s->q, 4 * sizeof(double));
@@ -414,14 +413,9 @@ prism_status write_state(prism_handle h, const prism_state* s) {
     std::memcpy(d.w, s->w, sizeof(d.w));
     std::memcpy(d.cov, s->cov, sizeof(d.cov));
     d.n_localised = s->n_localised;
-    // keep the anchor pose already on the device
-    CK(h, cudaStreamSynchronize(h->stream), "stream synchronize");
-    double anchor[7];
-    CK(h, cudaMemcpy(anchor, h->dstate->anchor_pose, sizeof(anchor), cudaMemcpyDeviceToHost), "read anchor pose");
-    std::memcpy(d.anchor_pose, anchor, sizeof(anchor));
-    CK(h, cudaMemcpy(h->dstate, &d, sizeof(d), cudaMemcpyHostToDevice), "write state");
-    PoseArg pa{};
-    LAUNCH(h, launch_prep(h->dstate, PREP_STATE, pa, h->stream), "pose matrices");
+    // the host frames of a step before are the caller's again
+    if (h->ev_in) CK(h, cudaEventSynchronize(h->ev_in), "previous host-frame copies");
+    LAUNCH(h, launch_set_state(h->dstate, d, h->stream), "state write");
     CK(h, cudaEventRecord(h->ev_state, h->stream), "state event");
     h->has_prior = false;
     h->anchor_at_mean = false;

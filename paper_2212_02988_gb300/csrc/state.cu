@@ -23,6 +23,29 @@ __global__ void k_prep(DevState* dev, int kind, PoseArg pose) {
     prep_mats_warp(dev, kind, pose);   // one warp
 }
 
+// A new state and its FP32 matrices; everything else of the device state but the
+// anchor's pose is cleared.  The state arrives as a kernel argument, so the call
+// neither waits for the stream nor copies: with the anchor's pose read back and
+// the struct written from the host (two copies and a wait, then k_prep) a
+// mapping loop over known poses idled for ~30 us a frame (16 frames of 251x189
+// into a 200^3 map, with the map's read-out and a view: 1026 -> 577 us).
+__global__ void __launch_bounds__(256) k_set_state(DevState* dev, const __grid_constant__ StateArg state) {
+    pdl_enter();
+    constexpr int kHead = offsetof(StateArg, n_localised) / 8, kAnchor = offsetof(DevState, anchor_pose) / 8;
+    static_assert(kHead == offsetof(DevState, pt) / 8 && sizeof(DevState) % 8 == 0, "the same head, whole words");
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    double* words = reinterpret_cast<double*>(dev);
+    for (int e = tid; e < (int)(sizeof(DevState) / 8); e += blockDim.x)
+        if (e < kAnchor || e >= kAnchor + 7) words[e] = e < kHead ? (&state.t[0])[e] : 0.0;
+    __syncthreads();
+    if (tid == 0) dev->n_localised = state.n_localised;
+    if (warp == 0) prep_mats_warp(dev, PREP_STATE, PoseArg{});
+}
+
+cudaError_t launch_set_state(DevState* dev, const StateArg& state, cudaStream_t s) {
+    return launch_pdl(k_set_state, 1, 256, s, dev, state);
+}
+
 cudaError_t launch_prep(DevState* dev, int kind, const PoseArg& pose, cudaStream_t s, bool pdl) {
     if (pdl) return launch_pdl(k_prep, 1, 32, s, dev, kind, pose);
     k_prep<<<1, 32, 0, s>>>(dev, kind, pose);
