@@ -2,6 +2,7 @@
 // body is in fuse_dev.cuh.
 #include "fuse_dev.cuh"
 #include "kernels.h"
+#include "render_dev.cuh"
 
 namespace prism {
 
@@ -9,10 +10,20 @@ namespace prism {
 // whose cells may read a voxel of them, to cells_list (ctr[1]).  rejected
 // (nullable): a nonzero value lists no tile (the localisation of this step was
 // rejected, so its frame is not fused).
+// depth (nullable): the observed frame whose depth validity the blocks past the
+// first cull_blocks write to mask.  The two are independent and short, and a
+// launch each costs a map update of known pose about 3 us of its 36 (200^3,
+// 251x189).
 __global__ void __launch_bounds__(256) k_fuse_cull(KParams P, const float* __restrict__ w2c, int* __restrict__ list,
                                                    int* __restrict__ cells_list, unsigned int* __restrict__ ctr,
-                                                   const int* __restrict__ rejected) {
+                                                   const int* __restrict__ rejected, int cull_blocks,
+                                                   const float* __restrict__ depth, uint8_t* __restrict__ mask) {
     pdl_enter();
+    if ((int)blockIdx.x >= cull_blocks) {
+        const int p = ((int)blockIdx.x - cull_blocks) * (int)blockDim.x + (int)threadIdx.x;
+        if (p < P.W * P.H) depth_mask_px(P, depth, mask, p);
+        return;
+    }
     __shared__ float sM[9], sb[3];
     load_w2c(w2c, sM, sb);
     __syncthreads();
@@ -58,14 +69,15 @@ static int fuse_grid() {
 }
 
 cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
-                               const float* rgb, const uint8_t* mask, DevStats* stats, int* list, int* cells_list,
-                               unsigned int* ctr, const int* rejected, cudaStream_t s) {
-    const int n = P.nbx * P.nby * P.nbz;
-    cudaError_t e = launch_pdl(k_fuse_cull, (n + 255) / 256, 256, s, P, w2c, list, cells_list, ctr, rejected);
+                               const float* rgb, uint8_t* mask, bool mask_ready, DevStats* stats, int* list,
+                               int* cells_list, unsigned int* ctr, const int* rejected, cudaStream_t s) {
+    const int cull = (P.nbx * P.nby * P.nbz + 255) / 256, pix = mask_ready ? 0 : (P.W * P.H + 255) / 256;
+    cudaError_t e = launch_pdl(k_fuse_cull, cull + pix, 256, s, P, w2c, list, cells_list, ctr, rejected, cull, depth,
+                               mask);
     if (e != cudaSuccess) return e;
-    if (P.bf16) return launch_pdl(k_fuse_list<true>, fuse_grid<true>(), 256, s, P, M, w2c, depth, rgb, mask, stats,
+    if (P.bf16) return launch_pdl(k_fuse_list<true>, fuse_grid<true>(), 256, s, P, M, w2c, depth, rgb, (const uint8_t*)mask, stats,
                                   (const int*)list, (const unsigned int*)ctr);
-    return launch_pdl(k_fuse_list<false>, fuse_grid<false>(), 256, s, P, M, w2c, depth, rgb, mask, stats,
+    return launch_pdl(k_fuse_list<false>, fuse_grid<false>(), 256, s, P, M, w2c, depth, rgb, (const uint8_t*)mask, stats,
                       (const int*)list, (const unsigned int*)ctr);
 }
 

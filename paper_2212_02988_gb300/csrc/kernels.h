@@ -136,10 +136,11 @@ cudaError_t launch_predict_prep(const KParams& P, DevState* dev, const double* i
 // cells_list the test also appends the tiles whose cells may read an updated
 // voxel to it, counted by ctr[1] (for launch_brick_flags).  Each list
 // has room for every tile.  rejected (device int, nullable;
-// DevState::rejected): nonzero lists no tile.
+// DevState::rejected): nonzero lists no tile.  mask_ready: `mask` holds the
+// frame's depth validity already; else the list's launch writes it.
 cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float* w2c, const float* depth,
-                               const float* rgb, const uint8_t* mask, DevStats* stats, int* list, int* cells_list,
-                               unsigned int* ctr, const int* rejected, cudaStream_t s);
+                               const float* rgb, uint8_t* mask, bool mask_ready, DevStats* stats, int* list,
+                               int* cells_list, unsigned int* ctr, const int* rejected, cudaStream_t s);
 
 // mapio.cu — fill with the prior, and conversion between the caller's dense
 // layout and the padded (ghost-bordered) device layout.

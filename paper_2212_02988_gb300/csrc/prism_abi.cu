@@ -508,11 +508,11 @@ prism_status do_localise(prism_handle h, const float* depth, const float* rgb, b
 
 prism_status do_fuse(prism_handle h, const float* depth, const float* rgb, bool mask_ready) {
     PhaseTimer t(h, PH_FUSE);
-    if (!mask_ready) LAUNCH(h, launch_depth_mask(h->kp, depth, h->o_mask, h->stream), "observation mask");
+    // (the frustum list's launch also evaluates the observation's mask where no localisation has)
     // after a localisation in the same step (mask_ready), a rejected step fuses nothing
     const size_t tiles = (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz;
     int* cells_list = h->kp.skip ? h->fuse_list + tiles : nullptr;
-    LAUNCH(h, launch_fuse_listed(h->kp, h->map, h->dstate->w2c, depth, rgb, h->o_mask, h->dstats, h->fuse_list,
+    LAUNCH(h, launch_fuse_listed(h->kp, h->map, h->dstate->w2c, depth, rgb, h->o_mask, mask_ready, h->dstats, h->fuse_list,
                                  cells_list, h->fuse_ctr, mask_ready ? &h->dstate->rejected : nullptr, h->stream),
            "fuse");
     ++h->launches;   // (two kernels: the frustum list and the update)
