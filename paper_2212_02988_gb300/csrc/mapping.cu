@@ -56,8 +56,9 @@ struct FrameLoss {
         D = obs_d[p];
         return true;
     }
-    __device__ __forceinline__ void get(int p, float d, const float* c, float& gd, float gc[3]) {
-        if (!(isfinite(D) && D > 0.0f)) return;
+    // (every ray is marched: the render's counters count the rays without a depth too)
+    __device__ __forceinline__ bool get(int p, float d, const float* c, float& gd, float gc[3]) {
+        if (!(isfinite(D) && D > 0.0f)) return false;
         const float r = d - D;
         gd = r * inv_sd2;
         ld = square(r, half_inv_sd2, loss);
@@ -67,6 +68,7 @@ struct FrameLoss {
             gc[k] = rc * inv_sc2;
             lc = lc + square(rc, half_inv_sc2, loss);
         }
+        return gd != 0.0f || gc[0] != 0.0f || gc[1] != 0.0f || gc[2] != 0.0f;
     }
 };
 

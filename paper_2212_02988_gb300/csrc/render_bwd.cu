@@ -24,11 +24,12 @@ struct GivenGradients {
         c2 = gC ? gC[3 * p + 2] : 0.0f;
         return gd != 0.0f || c0 != 0.0f || c1 != 0.0f || c2 != 0.0f;
     }
-    __device__ __forceinline__ void get(int, float, const float*, float& d, float c[3]) const {
+    __device__ __forceinline__ bool get(int, float, const float*, float& d, float c[3]) const {
         d = gd;
         c[0] = c0;
         c[1] = c1;
         c[2] = c2;
+        return true;   // (want)
     }
 };
 
