@@ -141,7 +141,9 @@ __device__ __forceinline__ void warp_scatter(const KParams& P, float* g_occ, flo
 // One 16x8-pixel tile (128 threads).  `loss` supplies the gradients: want(p)
 // says whether pixel p's ray is needed, get(p, d, c, gd, gc) gives
 // dL/d(depth) and dL/d(colour) of a hit rendered as (d, c) (passed only if
-// Loss::kImage) and returns whether any of them is not zero.  gpose: this thread's pose gradient (added to).  Returns the
+// Loss::kImage) and returns whether any of them is not zero.  gpose: this
+// thread's pose gradient (added to; of use only where get returns true for
+// every ray wanted).  Returns the
 // thread's hit sample index (0: none).
 template <bool BF16, bool DETAIL, int PX, class Loss>
 __device__ __forceinline__ int adjoint_tile(const KParams& P, const float* sR, const float* sc, const MapPlanes& M,
@@ -204,36 +206,34 @@ __device__ __forceinline__ int adjoint_tile(const KParams& P, const float* sR, c
 #pragma unroll
                     for (int k = 0; k < 3; ++k) c[k] = fmaf(alpha, col[1][k] - col[0][k], col[0][k]);
                 }
-                // a ray that takes no part carries nothing on: a zero gradient times a
-                // map value or slope that is not finite would be NaN
+                // (a ray that takes no part is not scattered: its zero gradient times a map
+                // value or slope that is not finite is NaN)
                 on = loss.get(p, d, c, gd, gc);
             }
-            if (on) {
-                float gA = gd * (ds[1] - ds[0]) * r.inv_n;
-                for (int c = 0; c < 3; ++c) gA += gc[c] * (col[1][c] - col[0][c]);
-                const float inv_df = 1.0f / (f[1] - f[0]);
-                const float gf[2] = {gA * (alpha - 1.0f) * inv_df, -gA * alpha * inv_df};
-                const float wa[2] = {1.0f - alpha, alpha};
-                const float rr[3] = {r.rx, r.ry, r.rz};
+            float gA = gd * (ds[1] - ds[0]) * r.inv_n;
+            for (int c = 0; c < 3; ++c) gA += gc[c] * (col[1][c] - col[0][c]);
+            const float inv_df = 1.0f / (f[1] - f[0]);
+            const float gf[2] = {gA * (alpha - 1.0f) * inv_df, -gA * alpha * inv_df};
+            const float wa[2] = {1.0f - alpha, alpha};
+            const float rr[3] = {r.rx, r.ry, r.rz};
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    g[m][0] = gf[m];
+            for (int m = 0; m < 2; ++m) {
+                g[m][0] = gf[m];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) g[m][1 + c] = gc[c] * wa[m];
-                    float gp[3];
+                for (int c = 0; c < 3; ++c) g[m][1 + c] = gc[c] * wa[m];
+                float gp[3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        gp[a] = gf[m] * go[m][a];
+                for (int a = 0; a < 3; ++a) {
+                    gp[a] = gf[m] * go[m][a];
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) gp[a] += gc[c] * wa[m] * gcol[m][c][a];
-                        gp[a] *= P.inv_vs32;
-                    }
-                    // dL/dt += gp; dL/dtheta += d (r x gp)
-                    gpose[0] += gp[0]; gpose[1] += gp[1]; gpose[2] += gp[2];
-                    gpose[3] += ds[m] * (rr[1] * gp[2] - rr[2] * gp[1]);
-                    gpose[4] += ds[m] * (rr[2] * gp[0] - rr[0] * gp[2]);
-                    gpose[5] += ds[m] * (rr[0] * gp[1] - rr[1] * gp[0]);
+                    for (int c = 0; c < 3; ++c) gp[a] += gc[c] * wa[m] * gcol[m][c][a];
+                    gp[a] *= P.inv_vs32;
                 }
+                // dL/dt += gp; dL/dtheta += d (r x gp)
+                gpose[0] += gp[0]; gpose[1] += gp[1]; gpose[2] += gp[2];
+                gpose[3] += ds[m] * (rr[1] * gp[2] - rr[2] * gp[1]);
+                gpose[4] += ds[m] * (rr[2] * gp[0] - rr[0] * gp[2]);
+                gpose[5] += ds[m] * (rr[0] * gp[1] - rr[1] * gp[0]);
             }
         }
     }

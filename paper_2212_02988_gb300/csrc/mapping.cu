@@ -10,39 +10,11 @@ namespace prism {
 
 namespace {
 
-// A sum of squares of FP32 values kept as an unevaluated pair h + l: each square
-// is exact (its rounding error by an FMA) and each addition keeps its rounding
-// error (Knuth's two-sum), so the pair is good to about 2^-46.  FP64 additions
-// (and conversions) cost ~64 cycles a warp instruction, these a dozen FP32 ones.
-struct Pair {
-    float h, l;
-};
-__device__ __forceinline__ Pair operator+(Pair a, Pair b) {
-    const float s = a.h + b.h, t = s - a.h;
-    const float e = ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l);
-    if (!isfinite(s)) return Pair{s, 0.0f};
-    const float h = s + e;
-    return Pair{h, e - (h - s)};
-}
-// Squares up to 1e36; larger values go to *big in FP64.
-__device__ __forceinline__ Pair square(float r, double scale, double* big) {
-    if (!(fabsf(r) < 1e18f)) {
-        atomicAdd(big, (double)r * (double)r * scale);
-        return Pair{0.0f, 0.0f};
-    }
-    const float h = r * r;
-    return Pair{h, fmaf(r, r, -h)};
-}
-__device__ __forceinline__ Pair warp_sum(Pair a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        a = a + Pair{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
-    return a;
-}
-
 // The loss of one rendered frame against its observation (obs_d, obs_c):
 // where the render hits and the observed depth is valid (finite, > 0),
-// (d - D)^2 / (2 sd^2) + |c - C|^2 / (2 sc^2).
+// (d - D)^2 / (2 sd^2) + |c - C|^2 / (2 sc^2), in FP64 (a hit's few FP64
+// instructions wait beside its gathers: pairs of floats were no faster, 178 us a
+// step of eight frames of 320x240 against 177).
 struct FrameLoss {
     static constexpr bool kImage = true;
     const float* obs_d;
@@ -51,7 +23,7 @@ struct FrameLoss {
     double half_inv_sd2, half_inv_sc2;
     double* loss;
     float D;
-    Pair ld, lc;
+    double l;   // this thread's loss
     __device__ __forceinline__ bool want(int p) {
         D = obs_d[p];
         return true;
@@ -61,13 +33,14 @@ struct FrameLoss {
         if (!(isfinite(D) && D > 0.0f)) return false;
         const float r = d - D;
         gd = r * inv_sd2;
-        ld = square(r, half_inv_sd2, loss);
+        double lc = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float rc = c[k] - obs_c[3 * p + k];
             gc[k] = rc * inv_sc2;
-            lc = lc + square(rc, half_inv_sc2, loss);
+            lc = fma((double)rc, (double)rc, lc);
         }
+        l = fma((double)r * (double)r, half_inv_sd2, lc * half_inv_sc2);
         return gd != 0.0f || gc[0] != 0.0f || gc[1] != 0.0f || gc[2] != 0.0f;
     }
 };
@@ -94,7 +67,7 @@ __global__ void __launch_bounds__(128) k_descent_frames(KParams P, const float* 
                                                         float* __restrict__ g_rgb, DevStats* __restrict__ stats) {
     pdl_enter();
     __shared__ float sR[9], sc[3];
-    __shared__ Pair s_l[2][4];
+    __shared__ double s_l[4];
     const size_t f = blockIdx.z, npix = (size_t)P.W * P.H;
     if (threadIdx.x < 12) {
         const float v = mats[12 * f + threadIdx.x];
@@ -106,25 +79,78 @@ __global__ void __launch_bounds__(128) k_descent_frames(KParams P, const float* 
     const int u = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7), v = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
     frame.obs_d += f * npix;
     frame.obs_c += 3 * f * npix;
-    frame.ld = frame.lc = Pair{0.0f, 0.0f};
+    frame.l = 0.0;
     float gpose[6] = {0, 0, 0, 0, 0, 0};   // (not used: known poses)
     int nsamp = 0;
     unsigned int uniq = 0;
     const int k = adjoint_tile<BF16, DETAIL, 0>(P, sR, sc, M, frame, g_occ, g_rgb, gpose, nsamp, uniq, blockIdx.x, blockIdx.y);
-    const Pair ld = warp_sum(frame.ld), lc = warp_sum(frame.lc);
-    if (lane == 0) {
-        s_l[0][warp] = ld;
-        s_l[1][warp] = lc;
-    }
+    double l = frame.l;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) s_l[warp] = l;
     if (stats) tile_stats<DETAIL>(stats, u < P.W && v < P.H, k >= 2, nsamp, uniq);
     __syncthreads();
     if (threadIdx.x == 0) {
-        const Pair a = (s_l[0][0] + s_l[0][1]) + (s_l[0][2] + s_l[0][3]);
-        const Pair b = (s_l[1][0] + s_l[1][1]) + (s_l[1][2] + s_l[1][3]);
-        const double l = ((double)a.h + (double)a.l) * frame.half_inv_sd2 + ((double)b.h + (double)b.l) * frame.half_inv_sc2;
+        l = (s_l[0] + s_l[1]) + (s_l[2] + s_l[3]);
         if (l != 0.0) atomicAdd(frame.loss, l);
     }
 }
+
+namespace {
+
+// A sum of squares of FP32 values, kept as an unevaluated sum of three floats
+// a + b + c: a square is h + l exactly (its rounding error by an FMA), and every
+// addition into a and b keeps its rounding error (Knuth's two-sum); only c's
+// additions round.  With b and c folded upwards once a row the sum is good to 1e-16
+// (against exact sums of 3 to 4,000 squares; FP64 additions: 1e-16 to 1e-14).  It takes
+// two dozen FP32 instructions a value where an FP64 conversion and FMA take 16
+// cycles each on an SM: a descent step on 128^3 voxels 86 us against 110, on 256^3
+// 430 against 536 (one and two frames).  The floats hold the squares of 2^-50
+// (below it l would underflow) to 1e14 (3e10 of them stay finite); `rest` sums the
+// others in FP64.
+struct SquareSum {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    double rest = 0.0;
+    // s = s + x with the rounding error left in x
+    static __device__ __forceinline__ void two_sum(float& s, float& x) {
+        const float t = s + x, z = t - s;
+        x = (s - (t - z)) + (x - z);
+        s = t;
+    }
+    __device__ __forceinline__ void add(float h, float l, float m) {
+        two_sum(a, h);
+        two_sum(b, h);
+        two_sum(b, l);
+        c += (h + l) + m;
+    }
+    __device__ __forceinline__ void square(float r) {
+        const float x = fabsf(r);
+        if (x <= 1e14f && (x >= 0x1p-50f || x == 0.0f)) {
+            const float h = r * r;
+            add(h, fmaf(r, r, -h), 0.0f);
+        } else {
+            rest = fma((double)r, (double)r, rest);
+        }
+    }
+    __device__ __forceinline__ void fold() {
+        two_sum(a, b);
+        two_sum(b, c);
+    }
+    // the floats summed over the N lanes that differ in the lowest bits
+    template <int N>
+    __device__ __forceinline__ void over_lanes() {
+#pragma unroll
+        for (int o = 1; o < N; o <<= 1)
+            add(__shfl_xor_sync(0xffffffffu, a, o), __shfl_xor_sync(0xffffffffu, b, o), __shfl_xor_sync(0xffffffffu, c, o));
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+    // this thread's rest, times scale, to *loss (rare)
+    __device__ __forceinline__ void add_rest(double scale, double* loss) const {
+        if (__double_as_longlong(rest)) atomicAdd(loss, rest * scale);
+    }
+};
+
+}  // namespace
 
 // The descent step on every padded element (ghosts included, each from the
 // voxel it clamps to, as the map load fills them):
@@ -140,10 +166,10 @@ __global__ void __launch_bounds__(256) k_map_step(KParams P, MapPlanes M, const 
                                                   float mu0_occ, float mu0_rgb, float inv_v0, double half_inv_v0,
                                                   double* loss) {
     pdl_enter();
-    __shared__ Pair part[8];
+    __shared__ float part[8][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t rows = P.npad / P.px;
-    Pair l{0.0f, 0.0f};
+    SquareSum l;
     for (uint32_t row = blockIdx.x * 8 + warp; row < rows; row += gridDim.x * 8) {
         const int gy = (int)(row % P.py) - 1, gz = (int)(row / P.py) - 1;
         const int y = min(max(gy, 0), P.ny - 1), z = min(max(gz, 0), P.nz - 1);
@@ -157,7 +183,7 @@ __global__ void __launch_bounds__(256) k_map_step(KParams P, MapPlanes M, const 
             {
                 const float m = map_load_rw<BF16>(M.occ, q);
                 const float dm = m - mu0_occ;
-                if (interior) l = l + square(dm, half_inv_v0, loss);
+                if (interior) l.square(dm);
                 map_store<BF16>(M.occ, q, m - lr_occ * (g_occ[i] + dm * inv_v0));
             }
             void* planes[3] = {M.r, M.g, M.b};
@@ -165,19 +191,27 @@ __global__ void __launch_bounds__(256) k_map_step(KParams P, MapPlanes M, const 
             for (int c = 0; c < 3; ++c) {
                 const float m = map_load_rw<BF16>(planes[c], q);
                 const float dm = m - mu0_rgb;
-                if (interior) l = l + square(dm, half_inv_v0, loss);
+                if (interior) l.square(dm);
                 map_store<BF16>(planes[c], q, m - lr_rgb * (g_rgb[3 * i + c] + dm * inv_v0));
             }
         }
+        l.fold();
     }
     __syncwarp();
-    l = warp_sum(l);
-    if (lane == 0) part[warp] = l;
+    l.add_rest(half_inv_v0, loss);
+    l.over_lanes<32>();
+    if (lane == 0) {
+        part[warp][0] = l.a;
+        part[warp][1] = l.b;
+        part[warp][2] = l.c;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += (double)part[w].h + (double)part[w].l;
-        atomicAdd(loss, s * half_inv_v0);
+    if (warp == 0) {
+        l.a = part[lane & 7][0];
+        l.b = part[lane & 7][1];
+        l.c = part[lane & 7][2];
+        l.over_lanes<8>();
+        if (lane == 0) atomicAdd(loss, l.value() * half_inv_v0);
     }
 }
 
