@@ -5,12 +5,13 @@
 
 namespace prism {
 
-// 6 blocks an SM (80 registers) with three samples' gathers in flight beat 8 (64)
-// here, where the longest rays set the time (8 in the rollouts, where the rate
-// does).  One block per 16x8 tile, block b rendering tile plan.order[b] (row-major without an order);
-// with plan.cost the block records the tile's cost for the next plan.
+// 5 blocks an SM (96 registers) with four samples' gathers in flight beat 6 with
+// three and 8 with two here, where the longest rays set the time (render_dev.cuh;
+// 8 in the rollouts, where the rate does).  One block per 16x8 tile, block b
+// rendering tile plan.order[b] (row-major without an order); with plan.cost the
+// block records the tile's cost for the next plan.
 template <bool BF16, bool DETAIL, int PX>
-__global__ void __launch_bounds__(128, DETAIL ? 10 : 6) k_render(KParams P, const float* __restrict__ mats, MapPlanes M,
+__global__ void __launch_bounds__(128, 5) k_render(KParams P, const float* __restrict__ mats, MapPlanes M,
                                                 float* __restrict__ depth, float* __restrict__ rgb,
                                                 uint8_t* __restrict__ mask, int32_t* __restrict__ hitk,
                                                 DevStats* __restrict__ stats, const double* __restrict__ anchor_src,
