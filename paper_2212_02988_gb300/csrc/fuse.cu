@@ -1,5 +1,7 @@
 // fuse.cu — single-stream launch of the per-voxel map update; the device
 // body is in fuse_dev.cuh.
+#include <cuda/atomic>
+
 #include "fuse_dev.cuh"
 #include "kernels.h"
 #include "render_dev.cuh"
@@ -31,20 +33,23 @@ __global__ void __launch_bounds__(256) k_fuse_cull(KParams P, const float* __res
 }
 
 // Persistent over the listed tiles (ctr[0] of them); a block reads its next
-// tile of the list beside the current one.  Bound by the latency of three
+// tile of the list beside the current one.  Without empty-space skipping nothing
+// reads the counters after it: the last block (ticket in ctr[1], which counts no
+// tiles then) clears them (a memset behind it: 12.3 us an update of a
+// 128^3 map from 320x240 against 10.9).  Bound by the latency of three
 // dependent rounds of loads (pixel, update decision, colours) at half the warps.
 template <bool BF16>
 __global__ void __launch_bounds__(256, 4) k_fuse_list(KParams P, MapPlanes M, const float* __restrict__ w2c,
                                                    const float* __restrict__ depth, const float* __restrict__ rgb,
                                                    const uint8_t* __restrict__ mask, DevStats* __restrict__ stats,
-                                                   const int* __restrict__ list, const unsigned int* __restrict__ ctr) {
+                                                   const int* __restrict__ list, unsigned int* __restrict__ ctr) {
     pdl_enter();
     __shared__ float sM[9], sb[3];
     __shared__ unsigned int s_count[2];
     load_w2c(w2c, sM, sb);
     if (threadIdx.x < 2) s_count[threadIdx.x] = 0u;
     __syncthreads();
-    const unsigned int count = ctr[0];
+    const unsigned int count = min(ctr[0], (unsigned int)(P.nbx * P.nby * P.nbz));   // (the list's room)
     int tile = blockIdx.x < count ? list[blockIdx.x] : 0;
     for (unsigned int i = blockIdx.x; i < count; i += gridDim.x) {
         const int cur = tile;
@@ -53,6 +58,10 @@ __global__ void __launch_bounds__(256, 4) k_fuse_list(KParams P, MapPlanes M, co
     }
     __syncthreads();
     add_fuse_counts(stats, s_count);
+    if (!P.skip && threadIdx.x == 0) {
+        cuda::atomic_ref<unsigned int, cuda::thread_scope_device> ticket(ctr[1]);
+        if (ticket.fetch_add(1u, cuda::memory_order_acq_rel) == gridDim.x - 1) ctr[0] = ctr[1] = 0u;
+    }
 }
 
 template <bool BF16>
@@ -76,9 +85,9 @@ cudaError_t launch_fuse_listed(const KParams& P, const MapPlanes& M, const float
                                mask);
     if (e != cudaSuccess) return e;
     if (P.bf16) return launch_pdl(k_fuse_list<true>, fuse_grid<true>(), 256, s, P, M, w2c, depth, rgb, (const uint8_t*)mask, stats,
-                                  (const int*)list, (const unsigned int*)ctr);
+                                  (const int*)list, ctr);
     return launch_pdl(k_fuse_list<false>, fuse_grid<false>(), 256, s, P, M, w2c, depth, rgb, (const uint8_t*)mask, stats,
-                      (const int*)list, (const unsigned int*)ctr);
+                      (const int*)list, ctr);
 }
 
 }  // namespace prism

@@ -73,15 +73,20 @@ __device__ __forceinline__ bool outside_frustum(const KParams& P, const float* s
     return out;
 }
 
-// t appended to `list` (count: its length) on the lanes that keep it; the
-// order is irrelevant.  Every thread of a warp calls it.
-__device__ __forceinline__ void append_kept(bool keep, int t, int* __restrict__ list, unsigned int* __restrict__ count) {
+// t appended to `list` (count: its length; room: how many it holds) on the lanes
+// that keep it; the order is irrelevant.  Every thread of a warp calls it.  The
+// count starts at zero (whoever reads the list last clears it), so the room is
+// never passed; the test keeps a count left behind by a call that failed from
+// becoming a write past the list.
+__device__ __forceinline__ void append_kept(bool keep, int t, int* __restrict__ list, unsigned int* __restrict__ count,
+                                            int room) {
     const unsigned int ballot = __ballot_sync(0xffffffffu, keep);
     const int lane = threadIdx.x & 31;
     unsigned int base = 0;
     if (lane == 0 && ballot) base = atomicAdd(count, (unsigned int)__popc(ballot));
     base = __shfl_sync(0xffffffffu, base, 0);
-    if (keep) list[base + __popc(ballot & ((1u << lane) - 1u))] = t;
+    const unsigned int at = base + __popc(ballot & ((1u << lane) - 1u));
+    if (keep && at < (unsigned int)room) list[at] = t;
 }
 
 // Tile t appended to `list` (count[0]) if it is in the frustum, and to
@@ -98,8 +103,8 @@ __device__ __forceinline__ void cull_tiles(const KParams& P, const float* sM, co
         keep = !outside_frustum(P, sM, sb, bx, by, bz, 1);
         cells = cells_list && !outside_frustum(P, sM, sb, bx, by, bz, 2);
     }
-    append_kept(keep, t, list, count);
-    if (cells_list) append_kept(cells, t, cells_list, count + 1);
+    append_kept(keep, t, list, count, n);
+    if (cells_list) append_kept(cells, t, cells_list, count + 1, n);
 }
 
 // The world-to-camera matrices into shared memory (12 threads; the caller

@@ -132,7 +132,8 @@ cudaError_t launch_predict_prep(const KParams& P, DevState* dev, const double* i
 // fuse.cu — the per-voxel map update with the world-to-camera matrices
 // `w2c` (12 FP32 on the device, DevState::w2c), in two launches: the frustum
 // test of every tile appends the tiles in view to `list`, then a persistent
-// grid updates only those; ctr[0] (zero between calls) counts them.  With
+// grid updates only those; ctr[0] (zero before the call; cleared by
+// launch_box_codes, or with P.skip = 0 by the update) counts them.  With
 // cells_list the test also appends the tiles whose cells may read an updated
 // voxel to it, counted by ctr[1] (for launch_brick_flags).  Each list
 // has room for every tile.  rejected (device int, nullable;

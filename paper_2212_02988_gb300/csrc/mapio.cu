@@ -147,7 +147,7 @@ template <bool BF16, int T>
 __global__ void __launch_bounds__(256) k_brick_flags(KParams P, MapPlanes M, const int* __restrict__ list,
                                                      const unsigned int* __restrict__ count) {
     pdl_enter();
-    const unsigned int n = list ? *count : (unsigned int)(P.nbx * P.nby * P.nbz);
+    const unsigned int all = P.nbx * P.nby * P.nbz, n = list ? min(*count, all) : all;   // (a list has room for all)
     for (unsigned int i = 2 * T * blockIdx.x; i < n; i += 2 * T * gridDim.x) {
         int tile[T];
 #pragma unroll

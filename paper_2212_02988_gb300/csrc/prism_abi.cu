@@ -145,6 +145,7 @@ struct prism_ctx {
     float* partials = nullptr;
     int* fuse_list = nullptr;
     unsigned int* fuse_ctr = nullptr;
+    bool fuse_dirty = false;   // a map update failed half-way: its list counters may not be zero
     unsigned int* counter = nullptr;
     // the anchor render's tile order (render_plan_block): the last anchor
     // render's tile costs and rotation, the planned order and its scratch,
@@ -512,6 +513,9 @@ prism_status do_fuse(prism_handle h, const float* depth, const float* rgb, bool 
     // after a localisation in the same step (mask_ready), a rejected step fuses nothing
     const size_t tiles = (size_t)h->kp.nbx * h->kp.nby * h->kp.nbz;
     int* cells_list = h->kp.skip ? h->fuse_list + tiles : nullptr;
+    // the update's last launch clears its list counters; a call that failed before it left them to this one
+    if (h->fuse_dirty) CK(h, cudaMemsetAsync(h->fuse_ctr, 0, 2 * sizeof(unsigned int), h->stream), "clear list counters");
+    h->fuse_dirty = true;
     LAUNCH(h, launch_fuse_listed(h->kp, h->map, h->dstate->w2c, depth, rgb, h->o_mask, mask_ready, h->dstats, h->fuse_list,
                                  cells_list, h->fuse_ctr, mask_ready ? &h->dstate->rejected : nullptr, h->stream),
            "fuse");
@@ -525,9 +529,8 @@ prism_status do_fuse(prism_handle h, const float* depth, const float* rgb, bool 
         }
         LAUNCH(h, launch_brick_flags(h->kp, h->map, cells_list, h->fuse_ctr + 1, h->stream), "brick flags");
         LAUNCH(h, launch_box_codes(h->kp, h->map, h->fuse_ctr, h->stream), "box codes");
-    } else {
-        CK(h, cudaMemsetAsync(h->fuse_ctr, 0, 2 * sizeof(unsigned int), h->stream), "clear list counters");
     }
+    h->fuse_dirty = false;
     return PRISM_OK;
 }
 
