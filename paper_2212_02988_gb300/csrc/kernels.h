@@ -195,6 +195,9 @@ cudaError_t launch_render_frames(const KParams& P, const float* mats, int frames
 // layout).  launch_map_step: mu <- mu - lr (g + (mu - mu0) / prior_var) on every
 // padded element of the occupancy and colour planes, the prior term of the loss
 // added to *loss; the empty-space index is left to the caller.
+// A batch's poses are the matrix kernel's argument (1.8 KB).  Batches of 8: 33 frames
+// of 320x240 take 629 us instead of 561, 64 of 80x60 235 instead of 134; of 64: 537
+// and 117, for an argument near the 4 KB limit.
 constexpr int kDescentBatch = 32;
 cudaError_t launch_descent_frames(const KParams& P, const double* poses, int frames, const MapPlanes& M,
                                   const float* obs_d, const float* obs_c, double sd, double sc, float* mats,

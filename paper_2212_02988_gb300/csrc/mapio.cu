@@ -245,15 +245,18 @@ cudaError_t launch_frame_upload(const float* s0, float* d0, size_t n0, const flo
 
 cudaError_t launch_brick_flags(const KParams& P, const MapPlanes& M, const int* list, const unsigned int* count,
                                cudaStream_t s) {
-    // one tile for each half of a block on small maps (a single wave, where the
-    // latency of one tile counts: the map-update phase of a 64^3 step 18.1 us
-    // against 20.1 with two), two on larger ones (a 256^3 step 91.4 against 92.5)
+    // One tile for each half of a block where latency counts: after a map update,
+    // whose list is a few waves at most (an update 15.0 us against 15.5 with two at
+    // 128^3, 15.9 against 17.4 at 160^3, 25.0 against 26.9 at 256^3), and over a whole
+    // map of up to 160^3 voxels (a load of its occupancy 13.6 against 14.4 at 128^3,
+    // 25.3 against 25.4 at 160^3).  Two over a larger map, where the rate counts (36.9
+    // against 36.0 at 192^3, 79.3 against 76.3 at 256^3).
     const int tiles = P.nbx * P.nby * P.nbz;
     auto go = [&](auto kern, int per) {
         const int need = (tiles + per - 1) / per;
         return launch_pdl(kern, need < 152 * 8 || !list ? need : 152 * 8, 256, s, P, M, list, count);
     };
-    if (tiles <= 4096) return P.bf16 ? go(k_brick_flags<true, 1>, 2) : go(k_brick_flags<false, 1>, 2);
+    if (list || tiles <= 8000) return P.bf16 ? go(k_brick_flags<true, 1>, 2) : go(k_brick_flags<false, 1>, 2);
     return P.bf16 ? go(k_brick_flags<true, 2>, 4) : go(k_brick_flags<false, 2>, 4);
 }
 
