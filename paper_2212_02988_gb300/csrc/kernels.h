@@ -30,7 +30,8 @@ enum PrepKind : int {
     PREP_AUX_REL = 2, // aux = pose argument -> anchor camera
     PREP_REL = 3,     // rel = Gauss-Newton pose -> anchor camera
     PREP_REL_NEXT = 4 // as PREP_REL with the state mean's pose as the anchor's (the
-                      // anchor rendered at the current mean, which may still be in flight)
+                      // anchor rendered at the current mean, which may still be in
+                      // flight); by the prediction only
 };
 
 // The six map planes (f32 or bf16 elements), each linear with a ghost border.

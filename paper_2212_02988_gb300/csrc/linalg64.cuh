@@ -94,15 +94,6 @@ __device__ __forceinline__ double so3_exp_jl_entry(const double w[3], bool exp, 
     return fma(s1, skew_entry(w, i, j), fma(s2, skew2_entry(w, th2, i, j), i == j ? 1.0 : 0.0));
 }
 
-// Entry (i, j) of J_l(w) = I + b K + c K^2, K = [w]_x (the same operations
-// whichever thread or kernel evaluates it).
-__device__ inline double so3_jl_entry(const double w[3], int i, int j) {
-    double a, b, c;
-    const double th2 = fdot3(w[0], w[0], w[1], w[1], w[2], w[2]);
-    so3_coeffs(th2, a, b, c);
-    return fma(b, skew_entry(w, i, j), fma(c, skew2_entry(w, th2, i, j), i == j ? 1.0 : 0.0));
-}
-
 // Entry (i, j) of the inverse left Jacobian of SO(3), I - K/2 + c K^2 with
 // c = 1/th^2 - (1 + cos th) / (2 th sin th); for th < 1/4 its Taylor series
 // 1/12 + th^2/720 + th^4/30240 + th^6/1209600 + th^8/47900160 (the same
@@ -221,42 +212,6 @@ __device__ __forceinline__ double warp_quat_exp_mul_unit(const double w[3], cons
     double rn = fma(-0.5, fma(n0, n0, fdot3(n1, n1, n2, n2, n3, n3)), 1.5);
     if (n0 < 0.0) rn = -rn;
     return (c == 0 ? n0 : (c == 1 ? n1 : (c == 2 ? n2 : n3))) * rn;
-}
-
-__device__ inline void mat3inv(const double* A, double* B) {
-    double c00 = A[4] * A[8] - A[5] * A[7], c01 = A[5] * A[6] - A[3] * A[8], c02 = A[3] * A[7] - A[4] * A[6];
-    double det = A[0] * c00 + A[1] * c01 + A[2] * c02;
-    double id = 1.0 / det;
-    B[0] = c00 * id;
-    B[1] = (A[2] * A[7] - A[1] * A[8]) * id;
-    B[2] = (A[1] * A[5] - A[2] * A[4]) * id;
-    B[3] = c01 * id;
-    B[4] = (A[0] * A[8] - A[2] * A[6]) * id;
-    B[5] = (A[2] * A[3] - A[0] * A[5]) * id;
-    B[6] = c02 * id;
-    B[7] = (A[1] * A[6] - A[0] * A[7]) * id;
-    B[8] = (A[0] * A[4] - A[1] * A[3]) * id;
-}
-
-// Unit quaternion (w >= 0) of a rotation matrix (Shepperd's method).
-__device__ inline void R_to_quat(const double* R, double* q) {
-    double tr = R[0] + R[4] + R[8], s;
-    if (tr > 0.0) {
-        s = 2.0 * sqrt(tr + 1.0);
-        q[0] = 0.25 * s; q[1] = (R[7] - R[5]) / s; q[2] = (R[2] - R[6]) / s; q[3] = (R[3] - R[1]) / s;
-    } else if (R[0] > R[4] && R[0] > R[8]) {
-        s = 2.0 * sqrt(1.0 + R[0] - R[4] - R[8]);
-        q[0] = (R[7] - R[5]) / s; q[1] = 0.25 * s; q[2] = (R[1] + R[3]) / s; q[3] = (R[2] + R[6]) / s;
-    } else if (R[4] > R[8]) {
-        s = 2.0 * sqrt(1.0 + R[4] - R[0] - R[8]);
-        q[0] = (R[2] - R[6]) / s; q[1] = (R[1] + R[3]) / s; q[2] = 0.25 * s; q[3] = (R[5] + R[7]) / s;
-    } else {
-        s = 2.0 * sqrt(1.0 + R[8] - R[0] - R[4]);
-        q[0] = (R[3] - R[1]) / s; q[1] = (R[2] + R[6]) / s; q[2] = (R[5] + R[7]) / s; q[3] = 0.25 * s;
-    }
-    double n = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    double sg = q[0] < 0.0 ? -1.0 : 1.0;
-    for (int i = 0; i < 4; ++i) q[i] = sg * q[i] / n;
 }
 
 // Rotation of a unit quaternion (value path; not the decision recipe).
@@ -432,73 +387,14 @@ __device__ __forceinline__ void warp_spd6_inverse(double a, bool* pd, double* ou
 // C = diag(Ra^T, Ra^T J_l(xi_theta)) mapping tangent steps to anchor-frame
 // perturbations, become (H' + L') y = -(g' + m) in y = C dxi, with
 // Ci = C^-1 = diag(Ra, J_l(xi_theta)^-1 Ra), L' = Ci^T L Ci and m = Ci^T L xi;
-// then dxi = Ci y.  One warp (all 32 lanes call it) computes, from Ra (3x3
-// row-major), L (6x6) and xi: ci1 = J_l(xi_theta)^-1 Ra (9), lp = L' (36,
-// row-major), m (6) and ji = J_l(xi_theta)^-1 (9).  scratch: 69 doubles of
-// shared memory.
-__device__ __forceinline__ void warp_gn_prior_terms(const double* Ra, const double* L, const double* xi, double* ci1,
-                                                    double* lp, double* m, double* ji, double* scratch) {
-    const int lane = threadIdx.x & 31;
-    double* Ji = scratch;         // J_l^-1 (9)
-    double* Ci = scratch + 9;     // diag blocks of Ci: Ra (9), J_l^-1 Ra (9)
-    double* T = scratch + 27;     // L Ci (36)
-    double* Lx = scratch + 63;    // L xi (6)
-    if (lane < 9) {
-        const double v = so3_jl_inv_entry(xi + 3, lane / 3, lane % 3);
-        Ji[lane] = v;
-        ji[lane] = v;
-    } else if (lane < 18) {
-        Ci[lane - 9] = Ra[lane - 9];
-    }
-    __syncwarp();
-    if (lane < 6) {
-        double lx = 0.0;
-        for (int k = 0; k < 6; ++k) lx = fma(L[6 * lane + k], xi[k], lx);
-        Lx[lane] = lx;
-    } else if (lane >= 8 && lane < 17) {   // J_l^-1 Ra
-        const int e = lane - 8, i = e / 3, j = e % 3;
-        const double v = fdot3(Ji[3 * i], Ra[j], Ji[3 * i + 1], Ra[3 + j], Ji[3 * i + 2], Ra[6 + j]);
-        Ci[9 + e] = v;
-        ci1[e] = v;
-    }
-    __syncwarp();
-    // T[k][j] = sum over the block of j: L[k][3 bj + l] Ci_bj[l][jj]; lanes 4..9 of the
-    // second round: m_i = sum over the block of i: Ci_bi[k][ii] (L xi)[3 bi + k]
-#pragma unroll
-    for (int round = 0; round < 2; ++round) {
-        const int e = lane + 32 * round;
-        const bool tm = e < 36, mm = round == 1 && lane >= 4 && lane < 10;
-        const int k = tm ? e / 6 : 0, j = tm ? e % 6 : 0, bj = j / 3, jj = j % 3;
-        const int i = mm ? lane - 4 : 0, bi = i / 3, ii = i % 3;
-        const double* Cb = Ci + 9 * (mm ? bi : bj);
-        const double a0 = mm ? Cb[ii] : L[6 * k + 3 * bj], a1 = mm ? Cb[3 + ii] : L[6 * k + 3 * bj + 1],
-                     a2 = mm ? Cb[6 + ii] : L[6 * k + 3 * bj + 2];
-        const double c0 = mm ? Lx[3 * bi] : Cb[jj], c1 = mm ? Lx[3 * bi + 1] : Cb[3 + jj],
-                     c2 = mm ? Lx[3 * bi + 2] : Cb[6 + jj];
-        const double v = fdot3(a0, c0, a1, c1, a2, c2);
-        if (tm) T[e] = v;
-        else if (mm) m[i] = v;
-    }
-    __syncwarp();
-    // L' = Ci^T T: L'[i][j] = sum over the block of i: Ci_bi[k][ii] T[3 bi + k][j]
-#pragma unroll
-    for (int round = 0; round < 2; ++round) {
-        const int e = lane + 32 * round;
-        if (round == 1 && e >= 36) break;
-        const int i = e / 6, j = e % 6, bi = i / 3, ii = i % 3;
-        const double* Cb = Ci + 9 * bi;
-        lp[e] = fdot3(Cb[ii], T[6 * (3 * bi) + j], Cb[3 + ii], T[6 * (3 * bi + 1) + j], Cb[6 + ii],
-                      T[6 * (3 * bi + 2) + j]);
-    }
-}
-
-// The same terms on two warps at once: warp_gn_prior_terms takes one warp
-// through both chains, 4,400 cycles, and the end of each Gauss-Newton pass
-// waited for it; the longer of these takes 2,900, as long as the next pass's
-// matrices beside it (localisation at 80x60 118.6 -> 113.5 us, at 640x480 123 ->
-// 121): _maps gives ci1, ji and L' (its lower triangle, mirrored),
-// _vector gives m.  The operations of each entry are those above.  scratch: 63
-// and 24 doubles.
+// then dxi = Ci y.  From Ra (3x3 row-major), L (6x6) and xi, one warp each (all
+// 32 lanes call them): _maps gives ci1 = J_l(xi_theta)^-1 Ra (9), lp = L' (36,
+// its lower triangle, mirrored) and ji = J_l(xi_theta)^-1 (9), _vector gives m (6).
+// scratch: 63 and 24 doubles of shared memory.  Two functions, because the
+// passes run them on two warps: one warp for both takes 4,400 cycles, and the
+// end of each pass waited for it; the longer of the two takes 2,900, as long as
+// the next pass's matrices beside it (localisation at 80x60 118.6 -> 113.5 us, at
+// 640x480 123 -> 121, each without its prediction).
 __device__ __forceinline__ void warp_gn_prior_maps(const double* Ra, const double* L, const double* xi, double* ci1,
                                                    double* lp, double* ji, double* scratch) {
     const int lane = threadIdx.x & 31;

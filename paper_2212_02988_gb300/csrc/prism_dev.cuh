@@ -118,7 +118,7 @@ struct DevState {
     // render-adjoint pose gradient (world-frame perturbation)
     double grad_pose[6];
     // The prior's terms of the current Gauss-Newton iterate in anchor-frame
-    // coordinates (linalg64.cuh, warp_gn_prior_terms), ready for the next
+    // coordinates (linalg64.cuh, warp_gn_prior_maps), ready for the next
     // pass's finish: Ci = diag(R_a, J_l(xi_theta)^-1 R_a) (two 3x3 blocks),
     // L' = Ci^T L Ci and m = Ci^T L xi (L = prior pose precision)
     double gn_Ci[18];

@@ -57,9 +57,9 @@ __device__ __forceinline__ double from_ordered(unsigned long long u) {
 }
 
 // The prediction on one block of 256 threads.  PREP = PREP_REL or
-// PREP_REL_NEXT: also what prep_mats_warp derives for that kind (the
+// PREP_REL_NEXT: also what prep_mats_warp derives for PREP_REL (the
 // Gauss-Newton start matrices of the new prior, whose iterate xi = 0 makes
-// J_l = I); PREP_NONE: not.
+// J_l = I), against the anchor's pose or the state mean's; PREP_NONE: not.
 //
 // What bounds it: FP64 instructions, ~64 cycles each on one SM sub-partition
 // whatever lanes are active, and the barriers between their chains.  So the
@@ -395,21 +395,20 @@ __device__ __forceinline__ void prep_mats_warp(DevState* dev, int kind, const Po
             warp_mats_rel(pose.p, dev->anchor_pose, dev->aux);
             break;
         default: {
-            // t[3] and q[4] are contiguous: the state mean's pose
-            const double* anchor = kind == PREP_REL_NEXT ? dev->t : dev->anchor_pose;
+            const double* anchor = dev->anchor_pose;
             warp_mats_rel(dev->cur_pose, anchor, dev->rel);
             // Ra (lanes 0..8), then the prior's terms of the iterate in anchor-frame
             // coordinates
             const double* qa = anchor + 3;
             const double v = quat_R_entry_rn(qa[0], qa[1], qa[2], qa[3], lane < 9 ? lane : 0);
-            __shared__ double s_ra[9], s_scr[69];
+            __shared__ double s_ra[9], s_scr[87];
             if (lane < 9) {
                 s_ra[lane] = v;
                 dev->gn_Ci[lane] = v;
             }
             __syncwarp();
-            warp_gn_prior_terms(s_ra, dev->prec_pp, dev->xi, dev->gn_Ci + 9, dev->gn_Lp, dev->gn_m, dev->gn_Ji,
-                                s_scr);
+            warp_gn_prior_maps(s_ra, dev->prec_pp, dev->xi, dev->gn_Ci + 9, dev->gn_Lp, dev->gn_Ji, s_scr);
+            warp_gn_prior_vector(s_ra, dev->prec_pp, dev->xi, dev->gn_m, s_scr + 63);
             // the localisation's constants: q0 = conj(q_anchor) (x) q_prior on
             // lanes 24..27, b0 = Ra^T (t_prior - t_anchor) on lanes 28..30
             const int c = lane & 3;

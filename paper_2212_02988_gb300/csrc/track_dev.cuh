@@ -603,7 +603,7 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
         // anchor-frame perturbation through C = T M = diag(Ra^T, Ra^T J_l(xi_theta)),
         // so the step solves (C^T H' C + L) dxi = -(C^T g' + L xi).  In y = C dxi
         // this is (H' + L') y = -(g' + m) with L' = Ci^T L Ci, m = Ci^T L xi and
-        // Ci = C^-1 = diag(Ra, J_l^-1 Ra), and dxi = Ci y (warp_gn_prior_terms):
+        // Ci = C^-1 = diag(Ra, J_l^-1 Ra), and dxi = Ci y (warp_gn_prior_maps):
         // the sums enter the FP64 solve with one addition each.  Ci, L' and m of
         // the current iterate were prepared by the previous pass's finish (or
         // with the start matrices before the first pass), off this pass's
@@ -716,7 +716,7 @@ __device__ __forceinline__ bool track_item(const KParams& P, const float* __rest
     // Sigma = (2 Ht + Mi^T L Mi)^-1 in world-frame perturbations, Mi =
     // diag(I, J_l(xi_theta)^-1).  With Ht = T Ht' T^T (T = diag(Ra, Ra), Ht' the
     // anchor-frame sum) and Mi^T L Mi = T L' T^T (L' = Ci^T L Ci of the final
-    // iterate, warp_gn_prior_terms), Sigma = T (2 Ht' + L')^-1 T^T: the sums
+    // iterate, warp_gn_prior_maps), Sigma = T (2 Ht' + L')^-1 T^T: the sums
     // enter the FP64 inverse with one FMA each, and the inverse is rotated once.
     const double* Lp = st + 170;
     const double* Ji = st + 206;
