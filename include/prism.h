@@ -230,7 +230,10 @@ prism_status prism_step_host(prism_handle h, const double* imu, int32_t n, doubl
  * PRISM_ENOTPD while the latest step's flags are raised). */
 prism_status prism_get_state(prism_handle h, prism_state* out);
 
-/* Replace the state (HOST pointer); the pending prior is discarded. */
+/* Replace the state (HOST pointer, read before the call returns); the pending
+ * prior is discarded.  The state is written in stream order: the call does not
+ * wait for the work enqueued before it (a failure of which a later call
+ * reports), only for the copies of a prism_step_host's frames still in flight. */
 prism_status prism_set_state(prism_handle h, const prism_state* s);
 
 /* Load / store the whole map in the linear caller layout (see Conventions):
@@ -350,7 +353,7 @@ prism_status prism_rollout(prism_handle h, int32_t n_seq, int32_t k, const doubl
  * poses: HOST, n x 7 (t, q); depth (n x H x W floats) and rgb (n x H x W x 3
  * floats): DEVICE.  sd, sc > 0; lr_occ, lr_rgb >= 0.  loss: HOST, 1 double,
  * the loss before the step (data and prior terms), or NULL; when given the
- * stream is synchronised.  The first call allocates the gradient and render
+ * stream is synchronised.  The first call allocates the gradient
  * buffers (PRISM_ENOMEM if it cannot).  PRISM_EINVAL for n < 1, a pose that
  * is not finite or has a zero quaternion, or a bad scale or step size. */
 prism_status prism_map_descent(prism_handle h, int32_t n, const double* poses, const float* depth,

@@ -393,8 +393,7 @@ __device__ __forceinline__ void warp_spd6_inverse(double a, bool* pd, double* ou
 // scratch: 63 and 24 doubles of shared memory.  Two functions, because the
 // passes run them on two warps: one warp for both takes 4,400 cycles, and the
 // end of each pass waited for it; the longer of the two takes 2,900, as long as
-// the next pass's matrices beside it (localisation at 80x60 118.6 -> 113.5 us, at
-// 640x480 123 -> 121, each without its prediction).
+// the next pass's matrices beside it.
 __device__ __forceinline__ void warp_gn_prior_maps(const double* Ra, const double* L, const double* xi, double* ci1,
                                                    double* lp, double* ji, double* scratch) {
     const int lane = threadIdx.x & 31;

@@ -89,8 +89,9 @@ cudaError_t launch_rollout_states(const KParams& P, const DevState* src, DevStat
 }
 
 // The render of many poses in one launch: grid z indexes the frame.  8 blocks
-// an SM: 7.18 ms for 320 frames of 640x480 against 7.39 ms at 6 and 12.2 ms
-// before the shared start of a warp's rays (render_dev.cuh).
+// an SM (64 registers): a call of 320 frames of 640x480 on a 256^3 map 8.67 ms (0.43
+// of them the states), 8.74, 8.90 and 9.19 ms with 7, 6 and 5; 15.2 ms before the
+// empty-space words and the shared start of a warp's rays (render_dev.cuh).
 template <bool BF16, int PX>
 __global__ void __launch_bounds__(128, 8) k_render_frames(KParams P, const float* __restrict__ mats, MapPlanes M,
                                                        float* __restrict__ depth, float* __restrict__ rgb,

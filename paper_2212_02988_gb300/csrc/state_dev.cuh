@@ -67,9 +67,10 @@ __device__ __forceinline__ double from_ordered(unsigned long long u) {
 // twelve in a row, one FMA a row of positions, none a row of velocities), the
 // independent chains (IMU statistics, quaternions and rotation, reciprocals,
 // noise terms, start matrices) run on warps of different sub-partitions, and
-// the window's sums share their shuffle trees: 11.4 us (35 with dense 12x12
-// products, five shuffles a sum and one warp's Cholesky with reciprocal square
-// roots).  The warp index is read from lane 0 so that the compiler knows the
+// the window's sums share their shuffle trees: 21 us alone with cold caches and 33
+// IMU rows (35 with dense 12x12 products, five shuffles a sum and one warp's
+// Cholesky with reciprocal square roots), 14.7 us a call in a loop of predictions
+// with their uploads (23.4).  The warp index is read from lane 0 so that the compiler knows the
 // branches on it to be warp-uniform: it otherwise takes every shuffle after
 // the first loop for a divergent one (~500 cycles each instead of 25; the
 // IMU statistics alone 16,800 cycles instead of 5,000).  The skipped products are by zeros: a covariance
