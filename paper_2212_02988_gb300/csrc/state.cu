@@ -20,7 +20,9 @@ __global__ void __launch_bounds__(256) k_predict_prep(KParams P, DevState* dev, 
 
 __global__ void k_prep(DevState* dev, int kind, PoseArg pose) {
     pdl_enter();
-    prep_mats_warp(dev, kind, pose);   // one warp
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);   // (warp-uniform to the compiler)
+    if (warp == 0) prep_mats_warp(dev, kind, pose);
+    else if (kind == PREP_REL) prep_vector_warp(dev);
 }
 
 // A new state and its FP32 matrices; everything else of the device state but the
@@ -47,8 +49,8 @@ cudaError_t launch_set_state(DevState* dev, const StateArg& state, cudaStream_t 
 }
 
 cudaError_t launch_prep(DevState* dev, int kind, const PoseArg& pose, cudaStream_t s, bool pdl) {
-    if (pdl) return launch_pdl(k_prep, 1, 32, s, dev, kind, pose);
-    k_prep<<<1, 32, 0, s>>>(dev, kind, pose);
+    if (pdl) return launch_pdl(k_prep, 1, 64, s, dev, kind, pose);
+    k_prep<<<1, 64, 0, s>>>(dev, kind, pose);
     return cudaGetLastError();
 }
 

@@ -381,7 +381,8 @@ __device__ __forceinline__ void predict_block(const KParams& P, DevState* dev, c
 // FP32 decision matrices of a pose (see PrepKind), computed once per pose by
 // the FP64 recipe so that no kernel block repeats the FP64 chain; for
 // PREP_REL also the Gauss-Newton tangent map of the current iterate (see
-// track_dev.cuh).  All 32 lanes of one warp call it; entries go one a lane.
+// track_dev.cuh), but for m (prep_vector_warp).  All 32 lanes of one warp call it;
+// entries go one a lane.
 __device__ __forceinline__ void prep_mats_warp(DevState* dev, int kind, const PoseArg& pose) {
     const int lane = threadIdx.x & 31;
     switch (kind) {
@@ -402,14 +403,13 @@ __device__ __forceinline__ void prep_mats_warp(DevState* dev, int kind, const Po
             // coordinates
             const double* qa = anchor + 3;
             const double v = quat_R_entry_rn(qa[0], qa[1], qa[2], qa[3], lane < 9 ? lane : 0);
-            __shared__ double s_ra[9], s_scr[87];
+            __shared__ double s_ra[9], s_scr[63];
             if (lane < 9) {
                 s_ra[lane] = v;
                 dev->gn_Ci[lane] = v;
             }
             __syncwarp();
             warp_gn_prior_maps(s_ra, dev->prec_pp, dev->xi, dev->gn_Ci + 9, dev->gn_Lp, dev->gn_Ji, s_scr);
-            warp_gn_prior_vector(s_ra, dev->prec_pp, dev->xi, dev->gn_m, s_scr + 63);
             // the localisation's constants: q0 = conj(q_anchor) (x) q_prior on
             // lanes 24..27, b0 = Ra^T (t_prior - t_anchor) on lanes 28..30
             const int c = lane & 3;
@@ -423,6 +423,17 @@ __device__ __forceinline__ void prep_mats_warp(DevState* dev, int kind, const Po
             if (lane >= 28 && lane < 31) dev->gn_b0[i2] = b0;
         }
     }
+}
+
+// PREP_REL's m = Ci^T L xi, on a warp beside prep_mats_warp's.
+__device__ __forceinline__ void prep_vector_warp(DevState* dev) {
+    const int lane = threadIdx.x & 31;
+    __shared__ double s_ra[9], s_scr[24];
+    const double* qa = dev->anchor_pose + 3;
+    const double v = quat_R_entry_rn(qa[0], qa[1], qa[2], qa[3], lane < 9 ? lane : 0);
+    if (lane < 9) s_ra[lane] = v;
+    __syncwarp();
+    warp_gn_prior_vector(s_ra, dev->prec_pp, dev->xi, dev->gn_m, s_scr);
 }
 
 }  // namespace prism
