@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(256) k_set_state(DevState* dev, const __grid_c
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     double* words = reinterpret_cast<double*>(dev);
     for (int e = tid; e < (int)(sizeof(DevState) / 8); e += blockDim.x)
-        if (e < kAnchor || e >= kAnchor + 7) words[e] = e < kHead ? (&state.t[0])[e] : 0.0;
+        if (e < kAnchor || e >= kAnchor + 7) words[e] = e < kHead ? reinterpret_cast<const double*>(&state)[e] : 0.0;
     __syncthreads();
     if (tid == 0) dev->n_localised = state.n_localised;
     if (warp == 0) prep_mats_warp(dev, PREP_STATE, PoseArg{});
